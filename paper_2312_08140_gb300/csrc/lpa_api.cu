@@ -482,6 +482,8 @@ lpa_status engine_create(Engine& E, int32_t G, const int64_t* vtx_off_h, const i
         float wmax = 0.f;
         memcpy(&wmax, &vr.max_weight_bits, sizeof(wmax));
         E.exact = true;
+        E.s.weight_bits = 1;
+        while (E.s.weight_bits < 32 && wmax >= (float)(1ull << E.s.weight_bits)) ++E.s.weight_bits;
         if (wmax <= 255.f && nnz > 0) {
             // one byte per entry: the float copy is converted, then freed
             unsigned char* w8 = nullptr;
@@ -546,7 +548,9 @@ lpa_status engine_view(Engine& E, const Engine& par, int32_t K, const lpa_config
 
 cudaError_t launch_bin(Engine& E, int mode, int bin, cudaStream_t st) {
     if (bin == 0) return launch_sweep_small(E.s, mode, st, E.sms);
-    if (bin == 1) return launch_sweep_warp(E.s, mode, st, E.sms);
+    if (bin == 1)
+        return (mode & ~kModeNonstrict) == MODE_ASYNC ? launch_sweep_warp(E.s, mode, st, E.sms)
+                                                      : launch_sweep_lane(E.s, mode, st, E.sms);
     return launch_sweep_block(E.s, mode, bin, E.sms, st);
 }
 

@@ -174,6 +174,7 @@ struct DevState {
     int32_t large_max;
     int32_t warp_slots;        // per-warp table slots = next pow2 >= 2 * warp_max
     int32_t block_slots[kBlockBins];   // per-block shared table slots of bins 2..4
+    int32_t weight_bits;       // integer weights: bits of the largest one (0: not known)
     int32_t dense_permille;    // dense sweep when entries of changed vertices >= this / 1000 of E
 };
 
@@ -215,7 +216,10 @@ cudaError_t launch_finalize(const DevState& s, cudaStream_t st, int sms);
 cudaError_t launch_set_params(Ctrl* ctrl, double tau, int max_iters, int mode, int nonstrict, int prune_other,
                               int32_t* labels_out, int local_ids, cudaStream_t st);
 cudaError_t launch_sweep_small(const DevState& s, int mode, cudaStream_t st, int sms);
+// Bin 1: a warp per vertex in the asynchronous mode, a lane per vertex in the
+// synchronous ones.
 cudaError_t launch_sweep_warp(const DevState& s, int mode, cudaStream_t st, int sms);
+cudaError_t launch_sweep_lane(const DevState& s, int mode, cudaStream_t st, int sms);
 // Block-per-vertex sweep of bin 2, 3 or 4 (one resident wave over `sms` SMs).
 // For bin 4 this also launches the partitioned rescan of overflowed rows.
 cudaError_t launch_sweep_block(const DevState& s, int mode, int bin, int sms, cudaStream_t st);

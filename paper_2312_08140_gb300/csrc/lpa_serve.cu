@@ -296,7 +296,8 @@ cudaError_t run_cycle(lpa_server* S) {
         // compaction: the cycle's frontier, then (async) the catch-up set
         e = launch_finish(s, mode, p == 0 ? kRoleStartSweep : kRoleCatchUp, none, 0, st, S->sms);
         if (e == cudaSuccess) e = launch_sweep_small(s, mode, st, S->sms);
-        if (e == cudaSuccess) e = launch_sweep_warp(s, mode, st, S->sms);
+        if (e == cudaSuccess)
+            e = mode == MODE_ASYNC ? launch_sweep_warp(s, mode, st, S->sms) : launch_sweep_lane(s, mode, st, S->sms);
         for (int b = 2; b < kBins && e == cudaSuccess; ++b)
             e = launch_sweep_block(s, mode, b, S->sms, st);
     }

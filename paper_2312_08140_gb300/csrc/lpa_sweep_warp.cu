@@ -1,59 +1,44 @@
-// lpa_sweep_warp.cu -- sweep for mid-degree vertices (small_max < d <= warp_max):
-// one warp per frontier vertex.
+// lpa_sweep_warp.cu -- asynchronous sweep for mid-degree vertices
+// (small_max < d <= warp_max): one warp per frontier vertex, so that a warp's
+// vertices are scanned one after another and read each other's new labels
+// (Sections 4.1, 4.1.1).  The synchronous modes take a lane per vertex
+// (lpa_sweep_lane.cu).
 //
 // The warp reads the row 32 entries at a time (coalesced index and weight
-// loads, one label gather per lane).  Within each 32-entry chunk, lanes that
-// hold the same label are grouped with __match_any_sync and their weights
-// combined (a popcount for unit weights, a group reduction for integer
-// weights), so each distinct label of the chunk costs one table update.
-//   d <= 32: the grouped sums are already the per-label totals K_{i->c}
-//            (Eq. 2) and the warp takes the argmax directly.
-//   d  > 32: group leaders add their sums into a per-warp open-addressing
-//            table in shared memory sized 2^ceil(log2(2d)) slots (so it can
-//            never fill) and list the slots they fill; the warp then scans
-//            the listed slots for the argmax and clears them.
+// loads, one label gather per lane).
+//   d <= 32: unit weights group the lanes that hold one label with
+//            __match_any_sync (the group's size is its total K_{i->c} of
+//            Eq. 2), integer weights are added up in the warp's table in
+//            shared memory, fp32 weights in lane order within each group;
+//            the warp takes the argmax of the totals.
+//   d  > 32: the labels' sums are added into the per-warp open-addressing
+//            table, sized 2^ceil(log2(2d)) slots (so it can never fill), and
+//            the slots a row fills are listed; the warp then scans the listed
+//            slots for the argmax and clears them.
 // A chunk whose labels all agree (after the first sweeps nearly every chunk)
 // skips the grouping: a row of one chunk takes that label's total directly,
 // and in a longer row such chunks extend a run of one label held in
 // registers, which reaches the table once.
+//
+// Integer weights once took the groups of __match_any_sync too, with
+// __reduce_add_sync per group: 64 + 129 cycles of an SM for 32 distinct
+// labels.  In the table a batch of 128 planted partitions (weights 1..4) runs
+// in 8.5 ms instead of 11.8; unit weights keep the groups (6.6 ms against 6.9).
 // Ties go to the smallest label id (Section 4.1.5); self-loops are skipped
 // (Algorithm 1).  On change, the warp re-reads the row and marks the
 // neighbours unprocessed (Section 4.1.4).
-#include "lpa_device.cuh"
+#include "lpa_warp_row.cuh"
 
 namespace lpa {
 
 constexpr int kWarpThreads = 256;
 constexpr int kWarpsPerBlock = kWarpThreads / 32;
-constexpr int kWarpUnroll = 3;      // chunks of 32 entries in flight per warp beyond the first
 constexpr unsigned kAsyncMinBatch = 16;       // async: at least this many consecutive visits per warp batch
 constexpr unsigned kAsyncMaxRunBatches = 8;   // async: batches a warp walks in one run
 constexpr unsigned kAsyncSmallRunBatches = 2;  // async, a bin of one wave of batches: batches per run
 constexpr unsigned kScatterWindow = 4096;   // batches per scattered window (a power of two)
 
-// Combined weight of the lanes in `peers` (all hold the same label).
-template <int WK>
-__device__ __forceinline__ typename Acc<WK>::T group_sum(unsigned peers, typename Acc<WK>::T w,
-                                                         int32_t lab, bool ok) {
-    if constexpr (WK == W_UNIT) {
-        return (typename Acc<WK>::T)__popc(peers);
-    } else if constexpr (WK == W_U32 || WK == W_U8) {
-        return __reduce_add_sync(peers, w);
-    } else {
-        // fp32: every lane of a group adds the group's weights in lane order,
-        // so all of them obtain the same value.
-        float sum = 0.f;
-        for (int q = 0; q < 32; ++q) {
-            float wq = __shfl_sync(kFull, w, q);
-            int32_t lq = __shfl_sync(kFull, lab, q);
-            if (ok && lq == lab) sum += wq;
-        }
-        (void)peers;
-        return sum;
-    }
-}
-
-template <bool ASYNC, int WK, bool BATCH, bool NS>
+template <int WK, bool BATCH, bool NS>
 __global__ void __launch_bounds__(kWarpThreads, 4) k_sweep_warp(DevState s, int flag_neighbours) {
     using T = typename Acc<WK>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -78,13 +63,12 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_sweep_warp(DevState s, int 
     const Labels L = labels_of(s);
     const bool marks = marks_on(s, flag_neighbours);
     const uint32_t sweep = NS ? (uint32_t)s.ctrl->iter + 1u : 0u;   // non-strict tie-break (Section 4.1.5)
-    const bool ident = identity_sweep<ASYNC, BATCH>(s);
-    const bool po = ASYNC && s.ctrl->prune_other != 0;               // FLPA's pruning rule
+    const bool po = s.ctrl->prune_other != 0;               // FLPA's pruning rule
     const unsigned cnt = bv.cnt;
     const unsigned nwarps = gridDim.x * kWarpsPerBlock;
     // each warp takes batches of B consecutive frontier entries (B <= 32) and
     // visits them one after another, B shrinking when the bin is too small to
-    // give every warp a full batch.  In the asynchronous mode B stays at least
+    // give every warp a full batch, but no further than
     // kAsyncMinBatch, so that a small graph is not scanned all at once (which
     // would make the pass synchronous).  On the 4313-vertex planted partition
     // of the tests, runs of 8 gave Q 0.731 where serial random orders reach
@@ -93,9 +77,9 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_sweep_warp(DevState s, int 
     // 16 stay within 0.02 of the serial median on every test graph in that
     // model, runs of 32 do not (ascending runs flood two of them).
     unsigned B = (cnt + nwarps - 1) / nwarps;
-    if (ASYNC && B < kAsyncMinBatch) B = kAsyncMinBatch;
+    if (B < kAsyncMinBatch) B = kAsyncMinBatch;
     B = B < 1u ? 1u : (B > 32u ? 32u : B);
-    // In the asynchronous mode the batches are visited in a scattered order
+    // The batches are visited in a scattered order
     // within windows of kScatterWindow batches (an odd multiplier modulo the
     // window's power-of-two size; the last, partial window in order).  In id
     // order, a graph spanning several waves of warps would have its low ids
@@ -104,20 +88,19 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_sweep_warp(DevState s, int 
     // blocks.  The windows keep the labels being gathered at a time to a few
     // graphs' worth (L2-resident) in large batches.
     const unsigned nbatch = (cnt + B - 1) / B;
-    // Asynchronous mode: a warp walks K consecutive batches in order (a run
+    // A warp walks K consecutive batches in order (a run
     // of K x B vertices), K as large as 8 while the bin still gives every
     // warp at least two runs; fewer runs in flight at once means fewer
     // vertices reading labels their neighbours are about to change (a
     // 140K-vertex planted partition inside a 4096-graph batch: median Q 0.645
     // with single batches, 0.750 with runs of 8, serial runs 0.745).
     unsigned K = 1;
-    if (ASYNC)
-        while (K < kAsyncMaxRunBatches && (unsigned long long)nbatch >= 2ull * (2u * K) * nwarps) K *= 2u;
+    while (K < kAsyncMaxRunBatches && (unsigned long long)nbatch >= 2ull * (2u * K) * nwarps) K *= 2u;
     // A bin of one wave (a small graph) has every batch in flight at once;
     // runs of two batches halve that (the twenty 100-5000-vertex test graphs,
     // 20 runs each on fresh handles: one run in 400 fell 0.02 below the
     // lowest of 16 serial orders with single batches, none with runs of two).
-    if (ASYNC && nbatch <= nwarps) K = kAsyncSmallRunBatches;
+    if (nbatch <= nwarps) K = kAsyncSmallRunBatches;
     const unsigned nruns = (nbatch + K - 1) / K;
     const unsigned full_windows = nruns / kScatterWindow;
     // Graphs kept in the caller's order inside a batch (the serving arena,
@@ -126,12 +109,12 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_sweep_warp(DevState s, int 
     // sweep, so the entries of a run are drawn at pseudo-random positions of
     // the frontier instead (a Feistel permutation, redrawn every sweep) --
     // what the shuffled storage order of batches gives the others.
-    const bool scatter_entries = ASYNC && BATCH && s.orig == nullptr;
+    const bool scatter_entries = BATCH && s.orig == nullptr;
     const uint64_t visit_seed = 0x2312081405ull + 0x9E3779B97F4A7C15ull * (uint64_t)s.ctrl->iter;
     unsigned long long my_changed = 0, my_changed_entries = 0;
     for (unsigned ri = blockIdx.x * kWarpsPerBlock + wib; ri < nruns; ri += nwarps) {
         unsigned pr = ri;
-        if (ASYNC && ri / kScatterWindow < full_windows)
+        if (ri / kScatterWindow < full_windows)
             pr = (ri & ~(kScatterWindow - 1u)) | ((ri * 0x9E3779B1u) & (kScatterWindow - 1u));
       for (unsigned pb = pr * K; pb < pr * K + K && pb < nbatch; ++pb) {
         const unsigned base = pb * B;
@@ -147,7 +130,7 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_sweep_warp(DevState s, int 
         if (okl) {
             stl = s.off[vl];
             enl = s.off_end[vl];
-            ownl = ASYNC ? __ldcg(L.C + vl) : L.C[vl];
+            ownl = __ldcg(L.C + vl);
             if constexpr (BATCH) {
                 if (s.done[s.gid[vl]]) actl = 0;
             }
@@ -167,7 +150,7 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_sweep_warp(DevState s, int 
             const int32_t vq = __shfl_sync(kFull, vl, q);
             const int64_t sq = __shfl_sync(kFull, stl, q);
             const bool ok = j != kEmptyKey && j != vq;
-            lab = ok ? (ident ? initial_label(s, j) : load_label<ASYNC>(L.C, j)) : kEmptyKey;
+            lab = ok ? load_label<true>(L.C, j) : kEmptyKey;
             w = ok ? load_weight<WK>(s.w, sq + lane) : (T)0;
         };
         int32_t j_cur = first_index(0), j_nxt = first_index(1);
@@ -200,7 +183,8 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_sweep_warp(DevState s, int 
                     if constexpr (WK == W_UNIT) {
                         sum = (T)__popc(__ballot_sync(kFull, ok));
                     } else if constexpr (WK == W_F32) {
-                        sum = group_sum<WK>(kFull, w_cur, lab_cur, ok);
+                        const unsigned okm = __ballot_sync(kFull, ok);
+                        sum = ordered_group_sum(okm, w_cur);
                     } else {
                         sum = __reduce_add_sync(kFull, w_cur);
                     }
@@ -209,29 +193,37 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_sweep_warp(DevState s, int 
                         cand = lmax;
                     }
                 } else {
-                    const unsigned peers = __match_any_sync(kFull, lab_cur);
-                    const T sum = group_sum<WK>(peers, w_cur, lab_cur, ok);
-                    if (ok && lane == (unsigned)(__ffs(peers) - 1)) {
-                        key = sum_key(sum);
-                        cand = lab_cur;
+                    T sum = (T)0;
+                    if constexpr (WK == W_UNIT || WK == W_F32) {
+                        const unsigned peers = __match_any_sync(kFull, lab_cur);
+                        if constexpr (WK == W_UNIT) sum = (T)__popc(peers);
+                        else sum = ordered_group_sum(ok ? peers : 0u, w_cur);
+                        if (ok) {
+                            key = sum_key(sum);
+                            cand = lab_cur;
+                        }
+                    } else {
+                        // integer weights meet in the table: grouping the lanes
+                        // and summing each group apart costs up to 193 cycles
+                        // of an SM for 32 distinct labels, two atomics about 4
+                        int slot = -1;
+                        if (ok) {
+                            slot = claim_slot(keys, ceil_log2((unsigned)wslots), lab_cur);
+                            if (slot < 0) atomicExch(&s.ctrl->error, 2);
+                            else atomicAdd(vals + slot, w_cur);
+                        }
+                        __syncwarp();
+                        if (slot >= 0) {
+                            key = sum_key(vals[slot]);
+                            cand = lab_cur;
+                        }
+                        __syncwarp();
+                        if (slot >= 0) {
+                            keys[slot] = kEmptyKey;
+                            vals[slot] = (T)0;
+                        }
+                        __syncwarp();
                     }
-                }
-            } else if (act && ident) {
-                // labels are the neighbour ids and occur once: a max over the row
-                unsigned long long bp = lab_cur != kEmptyKey ? pack_candidate(sum_key(w_cur), tr.key(lab_cur)) : 0ull;
-#pragma unroll 4
-                for (int64_t e = st + 32 + lane; e < en; e += 32) {
-                    const int32_t jj = load_index_keep(s.idx, e);
-                    if (jj != v) {
-                        const unsigned long long c =
-                            pack_candidate(sum_key(load_weight<WK>(s.w, e)), tr.key(initial_label(s, jj)));
-                        bp = c > bp ? c : bp;
-                    }
-                }
-                bp = warp_max_u64(bp);
-                if (lane == 0 && bp != 0ull) {
-                    key = (uint32_t)(bp >> 32);
-                    cand = tr.label(~(uint32_t)bp);
                 }
             } else if (act) {
                 const int log_slots = ceil_log2(2u * (unsigned)d);
@@ -265,7 +257,8 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_sweep_warp(DevState s, int 
                         if constexpr (WK == W_UNIT) {
                             sum = (T)__popc(__ballot_sync(kFull, ok));
                         } else if constexpr (WK == W_F32) {
-                            sum = group_sum<WK>(kFull, w, lab, ok);
+                            const unsigned okm = __ballot_sync(kFull, ok);
+                            sum = ordered_group_sum(okm, w);
                         } else {
                             sum = __reduce_add_sync(kFull, w);
                         }
@@ -279,9 +272,9 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_sweep_warp(DevState s, int 
                     flush_run();
                     bool ins = ok;
                     T add = w;
-                    if constexpr (WK != W_F32) {
+                    if constexpr (WK == W_UNIT) {
                         const unsigned peers = __match_any_sync(kFull, lab);
-                        add = group_sum<WK>(peers, w, lab, ok);
+                        add = (T)__popc(peers);
                         ins = ok && lane == (unsigned)(__ffs(peers) - 1);
                     }
                     insert_listed(ins, lab, add);
@@ -298,7 +291,7 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_sweep_warp(DevState s, int 
 #pragma unroll
                     for (int u = 0; u < kWarpUnroll; ++u) {
                         const bool ok = jj[u] != v;
-                        ll[u] = ok ? load_label<ASYNC>(L.C, jj[u]) : kEmptyKey;
+                        ll[u] = ok ? load_label<true>(L.C, jj[u]) : kEmptyKey;
                         wq[u] = ok ? load_weight<WK>(s.w, e0 + 32 * u + lane) : (T)0;
                     }
 #pragma unroll
@@ -340,12 +333,10 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_sweep_warp(DevState s, int 
             const int32_t best = best_key == 0xffffffffu ? -1 : tr.label(best_key);
             const bool changed = act && best >= 0 && best != own;   // warp-uniform
             const unsigned slot = __shfl_sync(kFull, pl, i);
-            if (lane == 0) record_label<ASYNC>(L, bv.chg + slot, v, own, best, changed);
-            if constexpr (ASYNC) {
-                // the next vertex's first-chunk labels were read before this
-                // update: lanes holding v as neighbour take its new label
-                if (changed && j_cur == v) lab_cur = best;
-            }
+            if (lane == 0) record_label<true>(L, bv.chg + slot, v, own, best, changed);
+            // the next vertex's first-chunk labels were read before this
+            // update: lanes holding v as neighbour take its new label
+            if (changed && j_cur == v) lab_cur = best;
             if (changed) {
                 if (marks) {
                     // FLPA's rule: a neighbour already carrying `best` stays unmarked
@@ -362,7 +353,7 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_sweep_warp(DevState s, int 
                             for (int u = 0; u < 4; ++u) f[u] = jj[u] != v ? __ldcg(s.flags + jj[u]) : (uint8_t)1;
 #pragma unroll
                             for (int u = 0; u < 4; ++u)
-                                if (f[u] == 0 && !(po && load_label<ASYNC>(L.C, jj[u]) == best)) s.flags[jj[u]] = 1;
+                                if (f[u] == 0 && !(po && load_label<true>(L.C, jj[u]) == best)) s.flags[jj[u]] = 1;
                         }
                     }
                 }
@@ -378,10 +369,10 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_sweep_warp(DevState s, int 
     flush_bin_counts(s, 1, my_changed, my_changed_entries);
 }
 
-template <bool ASYNC, int WK, bool BATCH, bool NS>
+template <int WK, bool BATCH, bool NS>
 static cudaError_t launch_warp_t(const DevState& s, int flag, cudaStream_t st, int sms) {
     const size_t smem = (size_t)kWarpsPerBlock * s.warp_slots * 9;     // table + list of filled slots
-    auto kern = k_sweep_warp<ASYNC, WK, BATCH, NS>;
+    auto kern = k_sweep_warp<WK, BATCH, NS>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     int per_sm = 0;
@@ -392,29 +383,23 @@ static cudaError_t launch_warp_t(const DevState& s, int flag, cudaStream_t st, i
     return cudaGetLastError();
 }
 
-template <bool ASYNC, bool BATCH, bool NS>
+template <bool BATCH, bool NS>
 static cudaError_t launch_warp_w(const DevState& s, int flag, cudaStream_t st, int sms) {
     switch (s.weight_kind) {
-        case W_UNIT: return launch_warp_t<ASYNC, W_UNIT, BATCH, NS>(s, flag, st, sms);
-        case W_U32: return launch_warp_t<ASYNC, W_U32, BATCH, NS>(s, flag, st, sms);
-        case W_U8: return launch_warp_t<ASYNC, W_U8, BATCH, NS>(s, flag, st, sms);
-        default: return launch_warp_t<ASYNC, W_F32, BATCH, NS>(s, flag, st, sms);
+        case W_UNIT: return launch_warp_t<W_UNIT, BATCH, NS>(s, flag, st, sms);
+        case W_U32: return launch_warp_t<W_U32, BATCH, NS>(s, flag, st, sms);
+        case W_U8: return launch_warp_t<W_U8, BATCH, NS>(s, flag, st, sms);
+        default: return launch_warp_t<W_F32, BATCH, NS>(s, flag, st, sms);
     }
 }
 
 template <bool NS>
-static cudaError_t launch_warp_ns(const DevState& s, bool async, int flag, cudaStream_t st, int sms) {
-    const bool batch = s.G > 1;
-    if (async) return batch ? launch_warp_w<true, true, NS>(s, flag, st, sms) : launch_warp_w<true, false, NS>(s, flag, st, sms);
-    return batch ? launch_warp_w<false, true, NS>(s, flag, st, sms) : launch_warp_w<false, false, NS>(s, flag, st, sms);
+static cudaError_t launch_warp_ns(const DevState& s, cudaStream_t st, int sms) {
+    return s.G > 1 ? launch_warp_w<true, NS>(s, 1, st, sms) : launch_warp_w<false, NS>(s, 1, st, sms);
 }
 
 cudaError_t launch_sweep_warp(const DevState& s, int mode, cudaStream_t st, int sms) {
-    const bool ns = (mode & kModeNonstrict) != 0;
-    mode &= ~kModeNonstrict;
-    const bool async = mode == MODE_ASYNC;
-    const int flag = mode != MODE_SYNC_FULL;
-    return ns ? launch_warp_ns<true>(s, async, flag, st, sms) : launch_warp_ns<false>(s, async, flag, st, sms);
+    return (mode & kModeNonstrict) ? launch_warp_ns<true>(s, st, sms) : launch_warp_ns<false>(s, st, sms);
 }
 
 }  // namespace lpa
