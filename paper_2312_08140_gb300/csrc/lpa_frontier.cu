@@ -10,6 +10,7 @@
 //   k_finalize     labels out (optionally as graph-local ids)
 //   k_validate     CSR checks at graph creation, weight exactness
 //   k_mod_*        modularity, Eq. 1 (Section 3.2), in fp64
+#include <algorithm>
 #include <vector>
 
 #include "lpa_device.cuh"
@@ -18,6 +19,7 @@ namespace lpa {
 
 constexpr int kFrontThreads = 256;
 constexpr int kVertsPerThread = 16;
+constexpr int kFinishVerts = 2048;      // vertices per block of k_finish, up to a full chip
 
 __global__ void k_set_params(Ctrl* ctrl, double tau, int max_iters, int mode, int nonstrict, int prune_other,
                              int32_t* labels_out, int local_ids) {
@@ -396,90 +398,139 @@ cudaError_t build_static_lists(DevState& s, cudaStream_t st, unsigned* counts, u
     return err;
 }
 
+// Sum over the lanes of a warp, the same in every lane.
+__device__ __forceinline__ long long warp_sum(long long x) {
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
+    return x;
+}
+
 // Run by the last block of k_finish once every block is done.  `rd` is the
 // buffer the pass just consumed; `wr` = rd ^ 1 received the next frontier
 // (or is dense; kRoleControl compacts nothing and keeps rd).  At the end of
 // sweep t (kRoleEndSweep, kRoleControl) it also runs the per-graph
 // convergence test of Algorithm 1 and sets the loop condition.
+//
+// Nothing else runs meanwhile, so its time is the latency of its loads: lane b
+// of the first warp owns bin b, every counter it needs is loaded at once, and
+// the totals are warp sums.  (One thread reading and writing the counters of
+// the five bins in turn took 12 of the 15 us that k_finish spent on a
+// 10,000-vertex graph.)
 __device__ void control_step(const DevState& s, int mode, int role, int dense_next, cudaGraphConditionalHandle h,
                              int in_graph) {
     Ctrl* c = s.ctrl;
     volatile Ctrl* vc = c;
-    const int t = vc->iter;
-    const int rd = vc->rd, wr = rd ^ 1;
-    int any = 0;
     const bool ends_sweep = role == kRoleEndSweep || role == kRoleControl;
     const bool compacted = role != kRoleControl;
+    const int b = (int)threadIdx.x;
+    const bool bin = b < kBins;
+    const int t = vc->iter;
+    const int rd = vc->rd, wr = rd ^ 1;
+    // this lane's bin, loaded before anything is waited for
+    long long cnt = 0, ent = 0, swv = 0, swe = 0, chg = 0, che = 0;
+    if (bin) {
+        cnt = vc->bin_cnt[rd][b];
+        ent = (long long)vc->bin_entries[rd][b];
+        swv = vc->sweep_bin_vertices[b];
+        swe = vc->sweep_bin_entries[b];
+        chg = (long long)vc->bin_changed[b];
+        che = (long long)vc->bin_changed_entries[b];
+    }
+    const double tau = vc->tau;
+    const int max_iters = vc->max_iters;
+    const int dense_rd = vc->dense[rd], cbuf = vc->cbuf, last_high = vc->last_pass_high, allow_dense = vc->allow_dense;
+    const unsigned long long pass_changed = vc->pass_changed_entries;
+    swv += cnt;                                       // the pass that just ended scanned buffer rd
+    swe += ent;
+    int any = 0;
     if (ends_sweep) {
-        const double tau = vc->tau;
-        const int max_iters = vc->max_iters;
-        unsigned long long changed_total = 0;
-        for (int b = 0; b < kBins; ++b) changed_total += vc->bin_changed[b];
+        __shared__ long long sh_changed;
+        if (threadIdx.x < 32) {
+            const long long sum = warp_sum(chg);
+            if (threadIdx.x == 0) sh_changed = sum;
+        }
+        __syncthreads();
+        const unsigned long long changed_total = (unsigned long long)sh_changed;
         for (int64_t g = threadIdx.x; g < s.G; g += blockDim.x) {
-            if (!s.done[g]) {
+            int done = s.done[g];
+            if (!done) {
                 const unsigned long long dn =
                     (s.G == 1) ? changed_total : ((volatile unsigned long long*)s.dN)[g];
                 const int it = s.iters[g] + 1;          // sweeps of graph g so far
+                const int64_t ng = s.g_end[g] - s.g_begin[g];
                 if (it <= kMaxHist) s.hist_changed[g * kMaxHist + it - 1] = (long long)dn;
                 s.iters[g] = it;
-                const int64_t ng = s.g_end[g] - s.g_begin[g];
                 if ((long long)dn <= dn_threshold(tau, ng)) {     // Algorithm 1: dN / N <= tau
-                    s.done[g] = 1;
+                    done = 1;
                     s.exit_reason[g] = 0;
                 } else if (it >= max_iters) {
-                    s.done[g] = 1;
+                    done = 1;
                     s.exit_reason[g] = 1;
                 }
+                if (done) s.done[g] = 1;
                 s.dN[g] = 0;
             }
-            any |= !s.done[g];
+            any |= !done;
         }
         any = __syncthreads_or(any);
     }
-    if (threadIdx.x != 0) return;
-    // the pass that just ended scanned buffer rd
-    for (int b = 0; b < kBins; ++b) {
-        c->sweep_bin_vertices[b] += vc->bin_cnt[rd][b];
-        c->sweep_bin_entries[b] += (long long)vc->bin_entries[rd][b];
-    }
+    if (threadIdx.x >= 32) return;
     if (ends_sweep) {
-        long long act = 0, scn = 0, che = 0;
-        for (int b = 0; b < kBins; ++b) {
-            act += vc->sweep_bin_vertices[b];
-            scn += vc->sweep_bin_entries[b];
-            che += (long long)vc->bin_changed_entries[b];
-        }
+        const long long act = warp_sum(swv), scn = warp_sum(swe), chs = warp_sum(che);
         if (t < kMaxHist) {
-            for (int b = 0; b < kBins; ++b) {
-                c->hist_bin_vertices[t][b] = vc->sweep_bin_vertices[b];
-                c->hist_bin_entries[t][b] = vc->sweep_bin_entries[b];
-                c->hist_bin_changed[t][b] = (long long)vc->bin_changed[b];
-                c->hist_bin_changed_entries[t][b] = (long long)vc->bin_changed_entries[b];
+            if (bin) {
+                c->hist_bin_vertices[t][b] = swv;
+                c->hist_bin_entries[t][b] = swe;
+                c->hist_bin_changed[t][b] = chg;
+                c->hist_bin_changed_entries[t][b] = che;
             }
-            c->hist_active[t] = act;
-            c->hist_scanned[t] = scn;
-            c->hist_changed_entries[t] = che;
+            if (b == 0) {
+                c->hist_active[t] = act;
+                c->hist_scanned[t] = scn;
+                c->hist_changed_entries[t] = chs;
+            }
         }
-        c->total_sweeps += 1;
-        c->total_scanned += scn;
-        // per pass: one launch per statically non-empty bin (the last bin adds
-        // the partitioned rescan), then the finish kernel
-        int per_pass = 1;
-        for (int b = 0; b < kBins; ++b) per_pass += s.bin_static[b] ? 1 : 0;
-        if (s.bin_static[kBins - 1] && s.ovf_possible) per_pass += 4;   // plan, slices, partitions, rescan
-        c->total_sweep_launches += mode == MODE_ASYNC ? 2 * per_pass : per_pass;
-        for (int b = 0; b < kBins; ++b) {
+        if (bin) {
             c->bin_changed[b] = 0;
             c->bin_changed_entries[b] = 0;
             c->sweep_bin_vertices[b] = 0;
             c->sweep_bin_entries[b] = 0;
         }
-        // a dense sync sweep wrote every scanned vertex into the other buffer
-        if (mode != MODE_ASYNC && vc->dense[rd]) c->cbuf ^= 1;
-        c->iter = t + 1;
-        c->any_active = any;
+        if (b == 0) {
+            // per pass: one launch per statically non-empty bin (the last bin adds
+            // the partitioned rescan), then the finish kernel
+            int per_pass = 1;
+            for (int q = 0; q < kBins; ++q) per_pass += s.bin_static[q] ? 1 : 0;
+            if (s.bin_static[kBins - 1] && s.ovf_possible) per_pass += 4;   // plan, slices, partitions, rescan
+            atomicAdd((unsigned long long*)&c->total_sweeps, 1ull);
+            atomicAdd((unsigned long long*)&c->total_scanned, (unsigned long long)scn);
+            atomicAdd((unsigned long long*)&c->total_sweep_launches,
+                      (unsigned long long)(mode == MODE_ASYNC ? 2 * per_pass : per_pass));
+            // a dense sync sweep wrote every scanned vertex into the other buffer
+            if (mode != MODE_ASYNC && dense_rd) c->cbuf = cbuf ^ 1;
+            c->iter = t + 1;
+            c->any_active = any;
+            // Marks are useless when the next pass is dense anyway.  After two
+            // sweeps in a row that changed almost every vertex, the next sweep
+            // skips them and the one after it is dense.  An asynchronous sweep's
+            // two passes count as one (its catch-up pass marks like its main pass).
+            const double changed = (double)pass_changed, active = (double)s.active_entries;
+            const bool high = changed * 1000.0 >= (double)kHighPermille * active;
+            bool skip = high && last_high;
+            // Synchronous labels do not depend on the frontier, so there a mark
+            // is only worth its store (and the sparse sweep its compaction) when
+            // the next frontier will be small.
+            if (mode != MODE_ASYNC && s.dense_permille <= 1000)
+                skip = skip || s.active_entries <= kDenseEntries ||
+                       changed * 1000.0 >= (double)s.dense_permille * active;
+            c->skip_marks = skip && allow_dense ? 1 : 0;
+            c->last_pass_high = high ? 1 : 0;
+            c->pass_changed_entries = 0;
+        }
+    } else if (bin) {
+        c->sweep_bin_vertices[b] = swv;
+        c->sweep_bin_entries[b] = swe;
     }
-    for (int b = 0; b < kBins; ++b) {
+    if (bin) {
         if (dense_next && compacted) {
             c->bin_cnt[wr][b] = s.bin_static[b];
             c->bin_entries[wr][b] = s.bin_static_entries[b];
@@ -488,25 +539,15 @@ __device__ void control_step(const DevState& s, int mode, int role, int dense_ne
         c->bin_entries[rd][b] = 0;
         c->row_next[b] = 0;
     }
-    if (ends_sweep) {
-        // Marks are useless when the next pass is dense anyway.  After two
-        // sweeps in a row that changed almost every vertex, the next sweep
-        // skips them and the one after it is dense.  An asynchronous sweep's
-        // two passes count as one (its catch-up pass marks like its main pass).
-        const bool high =
-            (double)vc->pass_changed_entries * 1000.0 >= (double)kHighPermille * (double)s.active_entries;
-        c->skip_marks = (high && vc->last_pass_high && vc->allow_dense) ? 1 : 0;
-        c->last_pass_high = high ? 1 : 0;
-        c->pass_changed_entries = 0;
+    if (b == 0) {
+        if (compacted) {
+            c->dense[wr] = dense_next;
+            c->rd = wr;
+        }
+        c->ovf_count = 0;
+        c->ticket = 0;
+        if (ends_sweep && in_graph) cudaGraphSetConditional(h, any ? 1u : 0u);
     }
-    if (compacted) {
-        c->dense[wr] = dense_next;
-        c->rd = wr;
-    }
-    c->ovf_count = 0;
-    c->ticket = 0;
-    __threadfence();
-    if (ends_sweep && in_graph) cudaGraphSetConditional(h, any ? 1u : 0u);
 }
 
 // After a pass over buffer rd: (1) at the end of a sparse sync sweep, apply
@@ -559,7 +600,8 @@ __global__ void __launch_bounds__(kFrontThreads) k_finish(DevState s, int mode, 
         // the main pass scanned every vertex (or recorded no marks): nothing
         // is left to reach in this sweep; the marks wait for the next one
     } else if (dense) {
-        if (mode != MODE_SYNC_FULL) {
+        // (a pass that wrote no marks leaves the flags clear)
+        if (mode != MODE_SYNC_FULL && !s.ctrl->skip_marks) {
             for (int64_t ch = gtid; ch < nchunks; ch += gstride) {
                 const int64_t v0 = ch * kVertsPerThread;
                 if (v0 + kVertsPerThread <= s.N) {
@@ -617,7 +659,10 @@ __global__ void __launch_bounds__(kFrontThreads) k_finish(DevState s, int mode, 
 
 cudaError_t launch_finish(const DevState& s, int mode, int role, cudaGraphConditionalHandle h, int in_graph,
                           cudaStream_t st, int sms) {
-    k_finish<<<sms * 4, kFrontThreads, 0, st>>>(s, mode, role, h, in_graph);
+    // a small graph takes few blocks: the last of them waits for the others
+    const int64_t want = (s.N + kFinishVerts - 1) / kFinishVerts;
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)sms * 4));
+    k_finish<<<blocks, kFrontThreads, 0, st>>>(s, mode, role, h, in_graph);
     return cudaGetLastError();
 }
 

@@ -23,6 +23,8 @@ constexpr int kBins = 5;                // thread / warp / 128-, 256-, 512-threa
 constexpr int kBlockBins = 3;           // bins 2..4 use the block kernel
 constexpr int kBlockThreads[kBlockBins] = {128, 256, 512};
 constexpr int kHighPermille = 900;      // "almost every vertex changed" (see skip_marks)
+constexpr long long kDenseEntries = 4 << 20;   // synchronous runs of graphs up to this many entries scan
+                                        // every vertex in every sweep
 constexpr int kSliceLen = 4096;         // entries per slice of an overflowing row
 constexpr int kMaxParts = 4096;         // partitions a row may use on the sliced path
 constexpr int kMaxSlices = 4096;        // slices a row may use on the sliced path (with the above: d <= 2^24)
