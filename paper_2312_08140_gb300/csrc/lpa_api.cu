@@ -131,6 +131,7 @@ struct Engine {
     unsigned* static_counts = nullptr;             // static-list scratch
     unsigned long long* static_ents = nullptr;
     unsigned long long* cap_scratch = nullptr;     // [3] overflow capacity sums
+    std::vector<void*> dom_scratch;                // majority kernels: bits, left-over slots
     std::vector<void*> ovf_scratch;                // sliced overflow path: pairs, counts, offsets
     int32_t* idx_owned = nullptr;
     bool borrowed = false;
@@ -190,6 +191,8 @@ void engine_free(Engine& E) {
     E.ovf = nullptr;
     for (void* p : E.ovf_scratch) E.owned.push_back(p);
     E.ovf_scratch.clear();
+    for (void* p : E.dom_scratch) E.owned.push_back(p);
+    E.dom_scratch.clear();
     pool_free_all(E.device, E.owned);
 }
 
@@ -199,9 +202,13 @@ lpa_status setup_blocks(Engine& E, cudaStream_t st) {
     std::vector<void*> old;
     if (E.ovf) old.push_back(E.ovf);
     for (void* p : E.ovf_scratch) old.push_back(p);
+    for (void* p : E.dom_scratch) old.push_back(p);
     pool_free_all(E.device, old);
     E.ovf = nullptr;
     E.ovf_scratch.clear();
+    E.dom_scratch.clear();
+    E.s.dom_bits = nullptr;
+    E.s.defer = nullptr;
     const size_t n = std::max<size_t>(E.s.bin_static[kBins - 1], 1);
     void* p = nullptr;
     cudaError_t err = pool_alloc(E.device, &p, n * sizeof(Overflow));
@@ -230,6 +237,22 @@ lpa_status setup_blocks(Engine& E, cudaStream_t st) {
     E.s.ovf_pairs_cap = pairs;
     E.s.ovf_cnt_cap = counts;
     E.s.ovf_possible = rows > 0 ? 1 : 0;
+    // majority kernels: single graphs with enough entries in the block bins
+    unsigned long long block_entries = 0;
+    for (int b = 2; b < kBins; ++b) block_entries += E.s.bin_static_entries[b];
+    if (E.s.G == 1 && block_entries >= (unsigned long long)kMajorityEntries) {
+        void* m[2] = {nullptr, nullptr};
+        const size_t mb[2] = {((size_t)E.s.N / 32 + 1) * sizeof(uint32_t), (size_t)E.s.N * sizeof(int32_t)};
+        for (int k = 0; k < 2; ++k) {
+            if (pool_alloc(E.device, &m[k], mb[k]) != cudaSuccess) {
+                cudaGetLastError();
+                return fail(LPA_ERR_OUT_OF_MEMORY, "majority scratch: %zu bytes", mb[k]);
+            }
+            E.dom_scratch.push_back(m[k]);
+        }
+        E.s.dom_bits = static_cast<uint32_t*>(m[0]);
+        E.s.defer = static_cast<int32_t*>(m[1]);
+    }
     return LPA_OK;
 }
 
@@ -367,6 +390,7 @@ lpa_status engine_create(Engine& E, int32_t G, const int64_t* vtx_off_h, const i
     E.s.N = n;
     E.s.E = nnz;
     E.s.G = G;
+    E.s.weight_max = 1.0f;
     E.weighted = weights != nullptr;
     E.borrowed = borrow;
     E.vtx_off_host.assign(vtx_off_h, vtx_off_h + G + 1);
@@ -473,6 +497,7 @@ lpa_status engine_create(Engine& E, int32_t G, const int64_t* vtx_off_h, const i
     // max-weight reduction over each row
     E.s.rows_distinct = (G == 1 && vr.desc_all == vr.desc_row_starts) ? 1 : 0;
 
+    if (weights) memcpy(&E.s.weight_max, &vr.max_weight_bits, sizeof(float));
     // weight representation: integer sums when every sum is an exact integer
     if (!weights) {
         E.exact = vr.c[5] == 0;
@@ -546,7 +571,13 @@ lpa_status engine_view(Engine& E, const Engine& par, int32_t K, const lpa_config
     return LPA_OK;
 }
 
-cudaError_t launch_bin(Engine& E, int mode, int bin, cudaStream_t st) {
+// `main`: the sweep's main pass, which the majority kernels precede (an
+// asynchronous catch-up pass is small).
+cudaError_t launch_bin(Engine& E, int mode, int bin, bool main, cudaStream_t st) {
+    if (main && E.s.dom_bits && bin >= 1) {
+        const cudaError_t err = launch_majority(E.s, mode, bin, st, E.sms);
+        if (err != cudaSuccess) return err;
+    }
     if (bin == 0) return launch_sweep_small(E.s, mode, st, E.sms);
     if (bin == 1)
         return (mode & ~kModeNonstrict) == MODE_ASYNC ? launch_sweep_warp(E.s, mode, st, E.sms)
@@ -567,11 +598,15 @@ int bin_at(int mode, int k) {
     return k;
 }
 
-cudaError_t enqueue_pass(Engine& E, int mode, cudaStream_t st) {
+cudaError_t enqueue_pass(Engine& E, int mode, bool main, cudaStream_t st) {
+    if (main && E.s.dom_bits) {
+        const cudaError_t err = launch_dominant(E.s, st, E.sms);
+        if (err != cudaSuccess) return err;
+    }
     for (int k = 0; k < kBins; ++k) {
         const int b = bin_at(mode, k);
         if (E.s.bin_static[b] == 0) continue;
-        cudaError_t err = launch_bin(E, mode, b, st);
+        cudaError_t err = launch_bin(E, mode, b, main, st);
         if (err != cudaSuccess) return err;
     }
     return cudaSuccess;
@@ -587,12 +622,12 @@ cudaError_t enqueue_pass(Engine& E, int mode, cudaStream_t st) {
 // `mode` may carry kModeNonstrict, which only the sweep kernels take.
 cudaError_t enqueue_sweep(Engine& E, int mode, cudaGraphConditionalHandle h, int in_graph, cudaStream_t st) {
     const int base = mode & ~kModeNonstrict;
-    cudaError_t err = enqueue_pass(E, mode, st);
+    cudaError_t err = enqueue_pass(E, mode, true, st);
     if (err != cudaSuccess) return err;
     if (base == MODE_ASYNC) {
         err = launch_finish(E.s, base, kRoleCatchUp, h, in_graph, st, E.sms);
         if (err != cudaSuccess) return err;
-        err = enqueue_pass(E, mode, st);
+        err = enqueue_pass(E, mode, false, st);
         if (err != cudaSuccess) return err;
     }
     return launch_finish(E.s, base, kRoleEndSweep, h, in_graph, st, E.sms);
@@ -783,10 +818,11 @@ lpa_status engine_run_profiled(Engine& E, int mode, double tol, int32_t max_iter
         float sweep_ms[kBins] = {0.f}, fin_ms = 0.f;
         const int passes = mode == MODE_ASYNC ? 2 : 1;
         for (int p = 0; p < passes; ++p) {
+            if (p == 0 && E.s.dom_bits) LPA_P(launch_dominant(E.s, st, E.sms));
             for (int k = 0; k < kBins; ++k) {
                 const int b = bin_at(mode, k);
                 LPA_P(cudaEventRecord(ev[k], st));
-                if (E.s.bin_static[b]) LPA_P(launch_bin(E, mode | (ns ? kModeNonstrict : 0), b, st));
+                if (E.s.bin_static[b]) LPA_P(launch_bin(E, mode | (ns ? kModeNonstrict : 0), b, p == 0, st));
             }
             LPA_P(cudaEventRecord(ev[kBins], st));
             LPA_P(launch_finish(E.s, mode, p + 1 < passes ? kRoleCatchUp : kRoleEndSweep, none, 0, st, E.sms));
@@ -866,7 +902,8 @@ lpa_status fill_props(const Engine& E, lpa_graph_props* p) {
     p->max_degree = E.max_degree;
     p->rows_distinct = E.s.rows_distinct;
     p->storage_order = E.order;
-    p->device_bytes = E.device_bytes + (int64_t)std::max<size_t>(E.s.bin_static[kBins - 1], 1) * sizeof(Overflow);
+    const int64_t dom_bytes = E.s.dom_bits ? (E.s.N / 32 + 1) * 4 + E.s.N * 4 : 0;
+    p->device_bytes = E.device_bytes + dom_bytes + (int64_t)std::max<size_t>(E.s.bin_static[kBins - 1], 1) * sizeof(Overflow);
     return LPA_OK;
 }
 

@@ -350,7 +350,9 @@ __device__ __forceinline__ void flush_bin_counts(const DevState& s, int bin, uns
 struct BinView {
     const int32_t* list;   // already offset to the bin's region
     int32_t* chg;          // sync-mode change marks, same offset
+    const int32_t* left;   // slots the majority kernels left over (null: every slot)
     unsigned cnt;
+    __device__ __forceinline__ unsigned slot(unsigned k) const { return left ? (unsigned)left[k] : k; }
 };
 
 __device__ __forceinline__ BinView bin_view(const DevState& s, int b) {
@@ -359,7 +361,9 @@ __device__ __forceinline__ BinView bin_view(const DevState& s, int b) {
     const int64_t base = s.bin_base[b];
     bv.list = (s.ctrl->dense[buf] ? s.slist : s.flist) + base;
     bv.chg = s.chg + base;
-    bv.cnt = s.ctrl->bin_cnt[buf][b];
+    const bool some = s.ctrl->dom_on && b >= 1;
+    bv.left = some ? s.defer + base : nullptr;
+    bv.cnt = some ? s.ctrl->defer_cnt[b] : s.ctrl->bin_cnt[buf][b];
     return bv;
 }
 
@@ -369,6 +373,8 @@ struct Labels {
     int32_t* C;
     int32_t* Cn;
     bool dense;
+    uint32_t* dom_bits;    // bit v set: vertex v carried dom_label when the pass began and has kept it
+    int32_t dom_label;     // (null and unused while no label dominates)
 };
 
 __device__ __forceinline__ Labels labels_of(const DevState& s) {
@@ -377,7 +383,17 @@ __device__ __forceinline__ Labels labels_of(const DevState& s) {
     L.C = s.lab[cb];
     L.Cn = s.lab[cb ^ 1];
     L.dense = s.ctrl->dense[s.ctrl->rd] != 0;
+    L.dom_bits = s.ctrl->dom_on ? s.dom_bits : nullptr;
+    L.dom_label = s.ctrl->dom_label;
     return L;
+}
+
+// Async: the new label of a vertex that changes.  A vertex that leaves the
+// dominating label loses its bit (one that joins it during the pass is found
+// through its label).
+__device__ __forceinline__ void write_label(const Labels& L, int32_t v, int32_t own, int32_t best) {
+    L.C[v] = best;
+    if (L.dom_bits != nullptr && own == L.dom_label) atomicAnd(L.dom_bits + (v >> 5), ~(1u << (v & 31)));
 }
 
 // Outcome of one scanned vertex.  Async: in-place write on change.  Sync,
@@ -388,7 +404,7 @@ template <bool ASYNC>
 __device__ __forceinline__ void record_label(const Labels& L, int32_t* chg_slot, int32_t v, int32_t own,
                                              int32_t best, bool changed) {
     if constexpr (ASYNC) {
-        if (changed) L.C[v] = best;
+        if (changed) write_label(L, v, own, best);
     } else {
         if (L.dense) {
             L.Cn[v] = changed ? best : own;

@@ -82,6 +82,7 @@ __global__ void k_init(DevState s) {
         c->dense[1] = 0;
         c->pass_changed_entries = 0;
         c->ovf_count = 0;
+        c->dom_on = 0;
         for (int b = 0; b < kBins; ++b) {
             c->row_next[b] = 0;
             c->bin_cnt[0][b] = s.bin_static[b];
@@ -501,10 +502,15 @@ __device__ void control_step(const DevState& s, int mode, int role, int dense_ne
             int per_pass = 1;
             for (int q = 0; q < kBins; ++q) per_pass += s.bin_static[q] ? 1 : 0;
             if (s.bin_static[kBins - 1] && s.ovf_possible) per_pass += 4;   // plan, slices, partitions, rescan
+            int majority = 0;               // once per sweep: sample, bits, one kernel per bin
+            if (s.dom_bits) {
+                majority = 2;
+                for (int q = 1; q < kBins; ++q) majority += s.bin_static[q] ? 1 : 0;
+            }
             atomicAdd((unsigned long long*)&c->total_sweeps, 1ull);
             atomicAdd((unsigned long long*)&c->total_scanned, (unsigned long long)scn);
             atomicAdd((unsigned long long*)&c->total_sweep_launches,
-                      (unsigned long long)(mode == MODE_ASYNC ? 2 * per_pass : per_pass));
+                      (unsigned long long)(majority + (mode == MODE_ASYNC ? 2 * per_pass : per_pass)));
             // a dense sync sweep wrote every scanned vertex into the other buffer
             if (mode != MODE_ASYNC && dense_rd) c->cbuf = cbuf ^ 1;
             c->iter = t + 1;
@@ -545,6 +551,7 @@ __device__ void control_step(const DevState& s, int mode, int role, int dense_ne
             c->rd = wr;
         }
         c->ovf_count = 0;
+        c->dom_on = 0;
         c->ticket = 0;
         if (ends_sweep && in_graph) cudaGraphSetConditional(h, any ? 1u : 0u);
     }

@@ -95,6 +95,10 @@ struct Ctrl {
     int32_t stall_copy;                  // test hook (lpa_graph_debug_stall): the block size of the
                                          // row kernel whose first block to produce a tile leaves that
                                          // tile's index copy unissued, once
+    int32_t dom_on;                      // a label dominates this pass (lpa_sweep_majority.cu)
+    int32_t dom_label;
+    unsigned int dom_next[kBins];        // majority kernels: next list position to take
+    unsigned int defer_cnt[kBins];       // rows they left to the ordinary kernels
     unsigned int row_next[kBins];        // block bins: next list position to take in this pass
     unsigned int row_next_pad[8 - kBins];
 };
@@ -163,6 +167,8 @@ struct DevState {
     int32_t* iters;            // [G]
     int32_t* exit_reason;      // [G]
     long long* hist_changed;   // [G * kMaxHist]
+    uint32_t* dom_bits;        // [N/32 + 1] bit v: vertex v carries the dominating label (null: no majority kernels)
+    int32_t* defer;            // [N] frontier slots the majority kernels left over, same bin regions
     struct Overflow* ovf;      // [bin_static[4]] last-bin rows whose labels overflowed the shared table
     uint2* ovf_pairs;          // sliced path: (label, sum bits) pairs grouped by partition per slice
     uint32_t* ovf_cnt;         // sliced path: pairs per (slice, partition)
@@ -176,6 +182,7 @@ struct DevState {
     int32_t large_max;
     int32_t warp_slots;        // per-warp table slots = next pow2 >= 2 * warp_max
     int32_t block_slots[kBlockBins];   // per-block shared table slots of bins 2..4
+    float weight_max;          // largest weight (1 for unit weights)
     int32_t weight_bits;       // integer weights: bits of the largest one (0: not known)
     int32_t dense_permille;    // dense sweep when entries of changed vertices >= this / 1000 of E
 };
@@ -222,6 +229,13 @@ cudaError_t launch_sweep_small(const DevState& s, int mode, cudaStream_t st, int
 // synchronous ones.
 cudaError_t launch_sweep_warp(const DevState& s, int mode, cudaStream_t st, int sms);
 cudaError_t launch_sweep_lane(const DevState& s, int mode, cudaStream_t st, int sms);
+// Majority kernels (lpa_sweep_majority.cu), for single graphs whose block bins
+// hold kMajorityEntries: launch_dominant looks for a label that dominates the
+// pass and marks its vertices; launch_majority then settles the rows of one bin
+// (1..4) that it decides and leaves the others to the bin's ordinary kernel.
+constexpr long long kMajorityEntries = 4 << 20;
+cudaError_t launch_dominant(const DevState& s, cudaStream_t st, int sms);
+cudaError_t launch_majority(const DevState& s, int mode, int bin, cudaStream_t st, int sms);
 // Block-per-vertex sweep of bin 2, 3 or 4 (one resident wave over `sms` SMs).
 // For bin 4 this also launches the partitioned rescan of overflowed rows.
 cudaError_t launch_sweep_block(const DevState& s, int mode, int bin, int sms, cudaStream_t st);

@@ -446,11 +446,14 @@ __global__ void __launch_bounds__(kLaneWarps * 32) k_sweep_lane(DevState s, int 
     const unsigned nchunks = (cnt + 31u) / 32u;
     const unsigned nwarps = gridDim.x * kLaneWarps;
     unsigned chunk = (unsigned)wib * gridDim.x + blockIdx.x;
-    auto vertex_of = [&](unsigned c) -> int32_t {
+    unsigned k_c = 0, k_n = 0;                      // their slots in the frontier list
+    auto vertex_of = [&](unsigned c, unsigned& slot) -> int32_t {
         const unsigned k = c * 32u + lane;
-        return c < nchunks && k < cnt ? bv.list[k] : -1;
+        if (c >= nchunks || k >= cnt) return -1;
+        slot = bv.slot(k);
+        return bv.list[slot];
     };
-    int32_t v_c = vertex_of(chunk), v_n = vertex_of(chunk + nwarps);
+    int32_t v_c = vertex_of(chunk, k_c), v_n = vertex_of(chunk + nwarps, k_n);
     int64_t st_c = 0, en_c = 0;
     int32_t done_c = 0;
     auto load_row = [&]() {
@@ -471,7 +474,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32) k_sweep_lane(DevState s, int 
         if (!full && chunk < nchunks) {
             // sort the chunk's vertices into the queues
             LaneRow r;
-            r.k = chunk * 32u + lane;
+            r.k = k_c;
             r.v = v_c;
             r.st = st_c;
             r.d = (int)(en_c - st_c);
@@ -494,7 +497,8 @@ __global__ void __launch_bounds__(kLaneWarps * 32) k_sweep_lane(DevState s, int 
             __syncwarp();
             chunk += nwarps;
             v_c = v_n;
-            v_n = vertex_of(chunk + nwarps);
+            k_c = k_n;
+            v_n = vertex_of(chunk + nwarps, k_n);
             load_row();
             continue;
         }

@@ -47,7 +47,7 @@
 // aggregating warps leave together at their next barrier, and the producing
 // warp leaves after its copies in flight have landed (again waited for with
 // a bound).  lpa_graph_debug_stall makes one copy go missing, to test this.
-#include "lpa_device.cuh"
+#include "lpa_warp_row.cuh"
 
 namespace lpa {
 
@@ -151,56 +151,6 @@ __device__ __forceinline__ bool mbar_wait_bounded_or(uint64_t* bar, unsigned par
     for (unsigned polls = 1;; ++polls) {
         if (mbar_try_wait(bar, parity)) return true;
         if ((polls & 63u) == 0 && (*stop || global_ns() - t0 > kWaitNs)) return false;
-    }
-}
-
-// Entries [e, e + 4) of idx (e a multiple of 4, e < en; idx starts at a
-// 16-byte aligned address): one 16-byte load where the vector lies inside the
-// row [st, en), else entry by entry; entries outside the row read as `fill`.
-__device__ __forceinline__ void load_idx4(const int32_t* idx, int64_t e, int64_t st, int64_t en, int32_t fill,
-                                          int32_t (&j)[4]) {
-    if (e >= st && e + 4 <= en) {
-        const int4 x = __ldg(reinterpret_cast<const int4*>(idx + e));
-        j[0] = x.x;
-        j[1] = x.y;
-        j[2] = x.z;
-        j[3] = x.w;
-    } else {
-        // the first or last vector of the row
-#pragma unroll
-        for (int c = 0; c < 4; ++c) j[c] = (e + c >= st && e + c < en) ? __ldg(idx + e + c) : fill;
-    }
-}
-
-// Marks the neighbours of changed vertex v unprocessed (Section 4.1.4): the
-// GROUP threads of rank 0..GROUP-1 walk row [st, en) in 4-entry vectors,
-// VEC vectors per thread in flight (their ids, then their flags, then the
-// stores).  FLPA's rule (po) leaves a neighbour already carrying `best`.
-template <bool ASYNC, int GROUP, int VEC>
-__device__ __forceinline__ void mark_row(const DevState& s, const Labels& L, int64_t st, int64_t en, int32_t v,
-                                         unsigned rank, bool po, int32_t best) {
-    for (int64_t e0 = (st & ~(int64_t)3) + 4 * (int64_t)rank; e0 < en; e0 += 4 * GROUP * VEC) {
-        int32_t j[VEC][4];
-        uint8_t f[VEC][4];
-#pragma unroll
-        for (int u = 0; u < VEC; ++u) {
-            const int64_t e = e0 + 4 * GROUP * u;
-            if (e < en) {
-                load_idx4(s.idx, e, st, en, v, j[u]);
-            } else {
-#pragma unroll
-                for (int c = 0; c < 4; ++c) j[u][c] = v;
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < VEC; ++u)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) f[u][c] = j[u][c] != v ? __ldcg(s.flags + j[u][c]) : (uint8_t)1;
-#pragma unroll
-        for (int u = 0; u < VEC; ++u)
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-                if (f[u][c] == 0 && !(po && load_label<ASYNC>(L.C, j[u][c]) == best)) s.flags[j[u][c]] = 1;
     }
 }
 
@@ -423,17 +373,20 @@ __global__ void __launch_bounds__(NT, RowsOccupancy<NT>::kBlocks) k_sweep_rows(D
     // the one after (nn_base, lane 0) are fetched a batch ahead; when a batch
     // starts, its rows' offsets and labels are loaded into `batch`.
     int32_t nxt_v = -1;
+    unsigned nxt_slot = 0;          // this lane's entry of the next batch: its slot in the frontier list
     unsigned nxt_base = 0, nn_base = 0;
     unsigned produced = 0;          // tiles produced by this block (index of the next one)
 
     auto list_at = [&](unsigned base) -> int32_t {
         const unsigned k = base + lane;
-        return (base < cnt && k < cnt) ? bv.list[k] : -1;
+        if (base >= cnt || k >= cnt) return -1;
+        nxt_slot = bv.slot(k);
+        return bv.list[nxt_slot];
     };
     auto start_batch = [&]() {      // warp 0: the batch at nxt_base becomes current
         RowMeta m;
         m.v = nxt_v;
-        m.k = nxt_base + lane;
+        m.k = nxt_slot;
         m.st = m.en = 0;
         m.own = 0;
         m.skip = 0;

@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_sweep_small_async(DevState s,
                 const int32_t own = sown[pos];
                 changed = best >= 0 && best != own;
                 if (changed) {
-                    L.C[v] = best;
+                    write_label(L, v, own, best);
                     if (marks) {
 #pragma unroll
                         for (int q = 0; q < MAXD; ++q) {

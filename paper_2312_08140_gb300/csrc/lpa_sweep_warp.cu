@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_sweep_warp(DevState s, int 
         // together so their latencies overlap.
         const unsigned kl = base + lane;
         const bool okl = lane < B && kl < cnt;
-        const unsigned pl = (scatter_entries && okl) ? shuffle_pos(kl, cnt, visit_seed) : kl;   // frontier slot
+        const unsigned pl = okl ? bv.slot(scatter_entries ? shuffle_pos(kl, cnt, visit_seed) : kl) : kl;   // frontier slot
         const int32_t vl = okl ? bv.list[pl] : 0;
         int64_t stl = 0, enl = 0;
         int32_t ownl = 0;

@@ -9,6 +9,56 @@ namespace lpa {
 
 constexpr int kWarpUnroll = 3;      // chunks of 32 entries in flight per warp beyond the first
 
+// Entries [e, e + 4) of idx (e a multiple of 4, e < en; idx starts at a
+// 16-byte aligned address): one 16-byte load where the vector lies inside the
+// row [st, en), else entry by entry; entries outside the row read as `fill`.
+__device__ __forceinline__ void load_idx4(const int32_t* idx, int64_t e, int64_t st, int64_t en, int32_t fill,
+                                          int32_t (&j)[4]) {
+    if (e >= st && e + 4 <= en) {
+        const int4 x = __ldg(reinterpret_cast<const int4*>(idx + e));
+        j[0] = x.x;
+        j[1] = x.y;
+        j[2] = x.z;
+        j[3] = x.w;
+    } else {
+        // the first or last vector of the row
+#pragma unroll
+        for (int c = 0; c < 4; ++c) j[c] = (e + c >= st && e + c < en) ? __ldg(idx + e + c) : fill;
+    }
+}
+
+// Marks the neighbours of changed vertex v unprocessed (Section 4.1.4): the
+// GROUP threads of rank 0..GROUP-1 walk row [st, en) in 4-entry vectors,
+// VEC vectors per thread in flight (their ids, then their flags, then the
+// stores).  FLPA's rule (po) leaves a neighbour already carrying `best`.
+template <bool ASYNC, int GROUP, int VEC>
+__device__ __forceinline__ void mark_row(const DevState& s, const Labels& L, int64_t st, int64_t en, int32_t v,
+                                         unsigned rank, bool po, int32_t best) {
+    for (int64_t e0 = (st & ~(int64_t)3) + 4 * (int64_t)rank; e0 < en; e0 += 4 * GROUP * VEC) {
+        int32_t j[VEC][4];
+        uint8_t f[VEC][4];
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) {
+            const int64_t e = e0 + 4 * GROUP * u;
+            if (e < en) {
+                load_idx4(s.idx, e, st, en, v, j[u]);
+            } else {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) j[u][c] = v;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < VEC; ++u)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) f[u][c] = j[u][c] != v ? __ldcg(s.flags + j[u][c]) : (uint8_t)1;
+#pragma unroll
+        for (int u = 0; u < VEC; ++u)
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if (f[u][c] == 0 && !(po && load_label<ASYNC>(L.C, j[u][c]) == best)) s.flags[j[u][c]] = 1;
+    }
+}
+
 // Words of a table slot: label, sum, and the lane mask of fp32 sums.
 template <int WK>
 constexpr int kTableWords = WK == W_F32 ? 3 : 2;
