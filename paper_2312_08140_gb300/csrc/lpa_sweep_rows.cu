@@ -10,8 +10,8 @@
 //
 //   * a row is cut into tiles of TILE = NC x P entries, NC the aggregating
 //     threads.  One warp produces the tile sequence of the block (rows taken
-//     from a per-bin counter in batches of 32, their metadata loaded by the
-//     32 lanes in parallel) up to kStages tiles ahead, and copies each tile's
+//     from a per-bin counter in batches of up to 32, their metadata loaded by
+//     the lanes in parallel) up to kStages tiles ahead, and copies each tile's
 //     neighbour ids into one of kStages shared-memory buffers with one bulk
 //     asynchronous copy (cp.async.bulk, completion counted on an mbarrier).
 //     In the 256- and 512-thread kernels the last warp only produces: it
@@ -51,7 +51,8 @@
 
 namespace lpa {
 
-constexpr int kRowBatch = 32;                  // rows taken from the counter at a time
+constexpr int kRowBatch = 32;                  // most rows taken from the counter at a time
+constexpr unsigned kBatchesPerBlock = 4;       // batches a block should get, so that blocks finish together
 constexpr int kStages = 4;                     // index buffers: a tile's copy starts three steps ahead
 constexpr int kSharedProbes = 16;              // probe bound of rows that may overflow the table
 constexpr unsigned long long kWaitNs = 2000000000ull;
@@ -272,6 +273,10 @@ __global__ void __launch_bounds__(NT, RowsOccupancy<NT>::kBlocks) k_sweep_rows(D
     const bool po = ASYNC && s.ctrl->prune_other != 0;               // FLPA's pruning rule
     const int log_S = ceil_log2((unsigned)S);
     const unsigned cnt = bv.cnt;
+    // Rows taken at a time: a few hundred hub rows in batches of 32 would keep
+    // a handful of the 152 blocks busy (R-MAT, 700,001 vertices: 211 rows of the
+    // last bin in 7 blocks).
+    const unsigned take = min((unsigned)kRowBatch, max(1u, cnt / (gridDim.x * kBatchesPerBlock)));
     const int64_t E_al = s.E & ~(int64_t)3;                          // end of the 16-byte aligned part of idx
 
     if (ident) {
@@ -368,7 +373,7 @@ __global__ void __launch_bounds__(NT, RowsOccupancy<NT>::kBlocks) k_sweep_rows(D
     }
 
     // ---- producer (warp 0) -----------------------------------------------------
-    // Rows come from the bin's counter in batches of kRowBatch.  The list
+    // Rows come from the bin's counter in batches of `take`.  The list
     // entries of the next batch (nxt_v, one per lane) and the counter value of
     // the one after (nn_base, lane 0) are fetched a batch ahead; when a batch
     // starts, its rows' offsets and labels are loaded into `batch`.
@@ -379,7 +384,7 @@ __global__ void __launch_bounds__(NT, RowsOccupancy<NT>::kBlocks) k_sweep_rows(D
 
     auto list_at = [&](unsigned base) -> int32_t {
         const unsigned k = base + lane;
-        if (base >= cnt || k >= cnt) return -1;
+        if (base >= cnt || k >= cnt || lane >= take) return -1;
         nxt_slot = bv.slot(k);
         return bv.list[nxt_slot];
     };
@@ -399,7 +404,7 @@ __global__ void __launch_bounds__(NT, RowsOccupancy<NT>::kBlocks) k_sweep_rows(D
         batch[lane] = m;
         nxt_base = __shfl_sync(kFull, nn_base, 0);
         nxt_v = list_at(nxt_base);
-        if (lane == 0) nn_base = atomicAdd(&s.ctrl->row_next[bin], (unsigned)kRowBatch);
+        if (lane == 0) nn_base = atomicAdd(&s.ctrl->row_next[bin], take);
         __syncwarp();
         if (lane == 0) {
             prod.bpos = 0;
@@ -413,7 +418,7 @@ __global__ void __launch_bounds__(NT, RowsOccupancy<NT>::kBlocks) k_sweep_rows(D
     auto produce = [&]() {
         for (;;) {                                     // warp-uniform: every lane reads the same state
             if (prod.exhausted || prod.pe < prod.pen) break;
-            if (prod.bpos >= kRowBatch) {
+            if (prod.bpos >= (int)take) {
                 start_batch();
                 if (prod.exhausted) break;
             }
@@ -477,10 +482,10 @@ __global__ void __launch_bounds__(NT, RowsOccupancy<NT>::kBlocks) k_sweep_rows(D
 
     if (wib == PW) {
         unsigned b0 = 0;
-        if (lane == 0) b0 = atomicAdd(&s.ctrl->row_next[bin], (unsigned)kRowBatch);
+        if (lane == 0) b0 = atomicAdd(&s.ctrl->row_next[bin], take);
         nxt_base = __shfl_sync(kFull, b0, 0);
         nxt_v = list_at(nxt_base);
-        if (lane == 0) nn_base = atomicAdd(&s.ctrl->row_next[bin], (unsigned)kRowBatch);
+        if (lane == 0) nn_base = atomicAdd(&s.ctrl->row_next[bin], take);
     }
     __syncthreads();                                   // mbarriers initialised, table clear
     __shared__ unsigned long long blk_changed, blk_changed_entries;   // this block's changes (thread 0)
