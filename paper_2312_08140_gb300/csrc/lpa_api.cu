@@ -575,7 +575,9 @@ lpa_status engine_view(Engine& E, const Engine& par, int32_t K, const lpa_config
 // asynchronous catch-up pass is small).
 cudaError_t launch_bin(Engine& E, int mode, int bin, bool main, cudaStream_t st) {
     if (main && E.s.dom_bits && bin >= 1) {
-        const cudaError_t err = launch_majority(E.s, mode, bin, st, E.sms);
+        cudaError_t err = cudaSuccess;
+        if ((mode & ~kModeNonstrict) == MODE_ASYNC && (bin == 2 || bin == 3)) err = launch_dominant(E.s, bin, st, E.sms);
+        if (err == cudaSuccess) err = launch_majority(E.s, mode, bin, st, E.sms);
         if (err != cudaSuccess) return err;
     }
     if (bin == 0) return launch_sweep_small(E.s, mode, st, E.sms);
@@ -600,7 +602,7 @@ int bin_at(int mode, int k) {
 
 cudaError_t enqueue_pass(Engine& E, int mode, bool main, cudaStream_t st) {
     if (main && E.s.dom_bits) {
-        const cudaError_t err = launch_dominant(E.s, st, E.sms);
+        const cudaError_t err = launch_dominant(E.s, 0, st, E.sms);
         if (err != cudaSuccess) return err;
     }
     for (int k = 0; k < kBins; ++k) {
@@ -818,7 +820,7 @@ lpa_status engine_run_profiled(Engine& E, int mode, double tol, int32_t max_iter
         float sweep_ms[kBins] = {0.f}, fin_ms = 0.f;
         const int passes = mode == MODE_ASYNC ? 2 : 1;
         for (int p = 0; p < passes; ++p) {
-            if (p == 0 && E.s.dom_bits) LPA_P(launch_dominant(E.s, st, E.sms));
+            if (p == 0 && E.s.dom_bits) LPA_P(launch_dominant(E.s, 0, st, E.sms));
             for (int k = 0; k < kBins; ++k) {
                 const int b = bin_at(mode, k);
                 LPA_P(cudaEventRecord(ev[k], st));

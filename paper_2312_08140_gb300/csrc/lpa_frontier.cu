@@ -506,6 +506,7 @@ __device__ void control_step(const DevState& s, int mode, int role, int dense_ne
             if (s.dom_bits) {
                 majority = 2;
                 for (int q = 1; q < kBins; ++q) majority += s.bin_static[q] ? 1 : 0;
+                if (mode == MODE_ASYNC) majority += (s.bin_static[2] ? 2 : 0) + (s.bin_static[3] ? 2 : 0);
             }
             atomicAdd((unsigned long long*)&c->total_sweeps, 1ull);
             atomicAdd((unsigned long long*)&c->total_scanned, (unsigned long long)scn);

@@ -234,7 +234,9 @@ cudaError_t launch_sweep_lane(const DevState& s, int mode, cudaStream_t st, int 
 // pass and marks its vertices; launch_majority then settles the rows of one bin
 // (1..4) that it decides and leaves the others to the bin's ordinary kernel.
 constexpr long long kMajorityEntries = 4 << 20;
-cudaError_t launch_dominant(const DevState& s, cudaStream_t st, int sms);
+// before_bin 0: at the start of a pass (any sweep but the first); 2, 3: before
+// that bin of an asynchronous pass (the first sweep only).
+cudaError_t launch_dominant(const DevState& s, int before_bin, cudaStream_t st, int sms);
 cudaError_t launch_majority(const DevState& s, int mode, int bin, cudaStream_t st, int sms);
 // Block-per-vertex sweep of bin 2, 3 or 4 (one resident wave over `sms` SMs).
 // For bin 4 this also launches the partitioned rescan of overflowed rows.

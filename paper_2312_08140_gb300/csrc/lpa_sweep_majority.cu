@@ -11,7 +11,9 @@
 // of a sweep's main pass:
 //
 //   k_dom_pick    samples 4096 entries' labels and finds the label, if any, that
-//                 holds 5/8 of them;
+//                 holds 5/8 of them (in the first asynchronous sweep, whose hubs
+//                 and low-degree vertices have their new labels by then, also
+//                 before the 128- and the 256-thread bin);
 //   k_dom_bits    sets bit v for each vertex v that carries it: 32 vertices per
 //                 word, so the array that the rows read is 1/32 of the labels
 //                 (8 MB for 67 M vertices, and largely L1 hits);
@@ -36,15 +38,18 @@ constexpr int kMajThreads = 256;
 constexpr int kMajLongThreads = 256;        // last bin: a block per row
 constexpr int kMajVec = 2;                  // 4-entry vectors per lane and step
 
-__global__ void __launch_bounds__(kPickThreads) k_dom_pick(DevState s) {
+// `mid`: between two bins of the first asynchronous sweep, where the bins before
+// have just left their own labels; otherwise before a later sweep.  The label
+// must hold `need` / 16 of the samples.
+__global__ void __launch_bounds__(kPickThreads) k_dom_pick(DevState s, int mid, int need) {
     __shared__ int ones[31], same;
     Ctrl* c = s.ctrl;
-    if (c->iter == 0) return;               // every label is still its vertex's own (dom_on is 0)
+    if ((c->iter == 0) != (mid != 0)) return;
     if (threadIdx.x < 31) ones[threadIdx.x] = 0;
     if (threadIdx.x == 31) same = 0;
     __syncthreads();
     const int32_t* C = s.lab[c->cbuf];
-    const uint64_t seed = (uint64_t)c->iter << 32;
+    const uint64_t seed = ((uint64_t)c->iter << 32) + ((uint64_t)need << 48);
     int32_t lab[kPickSamples];
 #pragma unroll
     for (int q = 0; q < kPickSamples; ++q) {
@@ -52,7 +57,8 @@ __global__ void __launch_bounds__(kPickThreads) k_dom_pick(DevState s) {
         lab[q] = __ldcg(C + __ldg(s.idx + e));
     }
     // a label that holds more than half of the samples has the majority's value
-    // in every bit
+    // in every bit (and most often one that holds a good part of them); the
+    // count below decides
     const unsigned lane = lane_id();
     for (int b = 0; b < 31; ++b) {
         int n = 0;
@@ -75,13 +81,13 @@ __global__ void __launch_bounds__(kPickThreads) k_dom_pick(DevState s) {
     }
     if (threadIdx.x == 0) {
         c->dom_label = label;
-        c->dom_on = 8 * same >= 5 * kPickThreads * kPickSamples ? 1 : 0;
+        c->dom_on = 16 * same >= need * kPickThreads * kPickSamples ? 1 : 0;
     }
 }
 
-__global__ void __launch_bounds__(256) k_dom_bits(DevState s) {
+__global__ void __launch_bounds__(256) k_dom_bits(DevState s, int mid) {
     const Ctrl* c = s.ctrl;
-    if (!c->dom_on) return;
+    if (!c->dom_on || (c->iter == 0) != (mid != 0)) return;
     const int32_t* C = s.lab[c->cbuf];
     const int32_t label = c->dom_label;
     const unsigned lane = lane_id();
@@ -103,11 +109,16 @@ __global__ void __launch_bounds__(256) k_dom_bits(DevState s) {
     }
 }
 
-cudaError_t launch_dominant(const DevState& s, cudaStream_t st, int sms) {
-    k_dom_pick<<<1, kPickThreads, 0, st>>>(s);
+// Before a sweep the label must hold 5/8 of the entries, before a row bin of the
+// first asynchronous sweep 3/8: the ordinary kernels gather at the rate of DRAM
+// sectors there, several times the cost of a bit that settles nothing.
+cudaError_t launch_dominant(const DevState& s, int before_bin, cudaStream_t st, int sms) {
+    const int mid = before_bin > 0;
+    const int need = mid ? 6 : 10;
+    k_dom_pick<<<1, kPickThreads, 0, st>>>(s, mid, need);
     const cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
-    k_dom_bits<<<sms * 8, 256, 0, st>>>(s);
+    k_dom_bits<<<sms * 8, 256, 0, st>>>(s, mid);
     return cudaGetLastError();
 }
 
