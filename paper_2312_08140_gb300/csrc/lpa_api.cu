@@ -877,10 +877,10 @@ lpa_status engine_modularity(Engine& E, int64_t v0, int64_t v1, const int32_t* l
         return LPA_OK;
     }
     LPA_CUDA(cudaMemsetAsync(E.Sigma, 0, (size_t)n * 8, st));
-    LPA_CUDA(cudaMemsetAsync(E.acc, 0, sizeof(ModAccum), st));
-    LPA_CUDA(launch_modularity(E.s, v0, v1, labels, E.Sigma, E.acc, st, E.sms));
+    LPA_CUDA(cudaMemsetAsync(E.acc, 0, kModAccumHead, st));
+    LPA_CUDA(launch_modularity(E.s, v0, v1, E.max_degree, labels, E.Sigma, E.acc, st, E.sms));
     ModAccum a;
-    LPA_CUDA(cudaMemcpyAsync(&a, E.acc, sizeof(a), cudaMemcpyDeviceToHost, st));
+    LPA_CUDA(cudaMemcpyAsync(&a, E.acc, kModAccumHead, cudaMemcpyDeviceToHost, st));
     LPA_CUDA(cudaStreamSynchronize(st));
     if (a.bad_label) return fail(LPA_ERR_INVALID_ARG, "%u labels outside [0, n)", a.bad_label);
     *q_out = a.two_m > 0.0 ? a.sigma / a.two_m - a.null_sum / (a.two_m * a.two_m) : 0.0;

@@ -945,18 +945,91 @@ cudaError_t launch_degree_hist(const DevState& s, unsigned long long* hist, cuda
 }
 
 // ------------------------------------------------------------ modularity --
-__device__ __forceinline__ double weight_f64(const DevState& s, int64_t e) {
-    if (s.weight_kind == W_UNIT) return 1.0;
-    if (s.weight_kind == W_U32) return (double)static_cast<const uint32_t*>(s.w)[e];
-    if (s.weight_kind == W_U8) return (double)static_cast<const unsigned char*>(s.w)[e];
-    return (double)static_cast<const float*>(s.w)[e];
+// Row sums: exact integers for unit and integer weights (below 2^31 per row,
+// checked at creation; the chip adds fp64 at 1/64 of its integer rate), fp64
+// for fp32 weights.
+template <int WK>
+using ModSum = typename std::conditional<WK == W_F32, double, unsigned long long>::type;
+
+template <int WK>
+__device__ __forceinline__ ModSum<WK> mod_weight(const DevState& s, int64_t e) {
+    if constexpr (WK == W_UNIT) return 1ull;
+    else if constexpr (WK == W_U32) return (unsigned long long)__ldcs(static_cast<const uint32_t*>(s.w) + e);
+    else if constexpr (WK == W_U8) return (unsigned long long)__ldg(static_cast<const unsigned char*>(s.w) + e);
+    else return (double)__ldcs(static_cast<const float*>(s.w) + e);
 }
 
-// One warp per vertex i of [v0, v1): K_i, and the weight of entries whose two
-// ends share a label (sigma); Sigma_c += K_i.
-__global__ void k_mod_rows(DevState s, int64_t v0, int64_t v1, const int32_t* labels, double* Sigma,
-                           ModAccum* acc) {
+// Four consecutive ids [a, a + 4) (a a multiple of 4); those outside [st, en)
+// read as `fill`.  `vec`: idx starts on a 16-byte boundary.
+__device__ __forceinline__ void mod_ids(const int32_t* idx, int64_t a, int64_t st, int64_t en, int64_t E, bool vec,
+                                        int32_t fill, int32_t (&j)[4]) {
+    if (vec && a + 4 <= E && a < en) {
+        const int4 x = __ldcs(reinterpret_cast<const int4*>(idx + a));
+        const int32_t z[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) j[c] = a + c >= st && a + c < en ? z[c] : fill;
+    } else {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) j[c] = a + c >= st && a + c < en ? __ldcs(idx + a + c) : fill;
+    }
+}
+
+// Adds to K the weights, and to sg the weights of entries whose other end has
+// label ci, of this thread's share of entries [e0, en) of a row starting at
+// st: 4-entry vectors, two in flight, thread `rank` of GROUP.
+template <int GROUP, int WK>
+__device__ __forceinline__ void mod_walk(const DevState& s, const int32_t* labels, int64_t v0, int64_t nloc, int64_t e0,
+                                         int64_t st, int64_t en, int32_t ci, bool vec, unsigned rank,
+                                         ModSum<WK>& K, ModSum<WK>& sg) {
+    for (int64_t a = (e0 & ~(int64_t)3) + 4 * (int64_t)rank; a < en; a += 8 * GROUP) {
+        int32_t j[2][4], l[2][4];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) mod_ids(s.idx, a + 4 * GROUP * u, e0 > st ? e0 : st, en, s.E, vec, -1, j[u]);
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                // labels are given in the caller's vertex order
+                const int64_t q = j[u][c] >= 0 ? (int64_t)initial_label(s, j[u][c]) - v0 : -1;
+                l[u][c] = q >= 0 && q < nloc ? __ldg(labels + q) : -1;
+            }
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if (j[u][c] >= 0) {
+                    const ModSum<WK> w = mod_weight<WK>(s, a + 4 * GROUP * u + c);
+                    K += w;
+                    if (l[u][c] == ci) sg += w;
+                }
+    }
+}
+
+// K_i of the vertices i of [v0, v1), added up per community in Sigma, and the
+// weight of entries whose two ends share a label (sigma).  A warp takes `width`
+// consecutive vertices: short rows a lane each (an instruction then serves 32
+// rows; a warp per row left most lanes of a short row idle), longer ones with
+// all its lanes, and rows beyond kModLong entries are listed for k_mod_long, so
+// that a hub does not hold up one warp.  Communities are few and large where it
+// matters, so the warp first adds up the K_i that share the batch's first label,
+// and the block keeps sums in a small shared cache: adding every K_i to Sigma by itself serialised on
+// the hot communities (2 M vertices of an R-MAT graph, nearly all in one
+// community: 7.5 ms).
+constexpr int kModThreads = 256;
+constexpr int kModSlots = 256;          // labels cached per block
+constexpr int kModShort = 64;           // longest row a lane takes
+
+template <int WK>
+__global__ void __launch_bounds__(kModThreads) k_mod_rows(DevState s, int64_t v0, int64_t v1, const int32_t* labels,
+                                                          double* Sigma, ModAccum* acc, int width, int vec) {
     __shared__ double sh_two_m, sh_sigma;
+    __shared__ int32_t ckey[kModSlots];
+    using T = ModSum<WK>;
+    __shared__ T cval[kModSlots];
+    for (int q = threadIdx.x; q < kModSlots; q += blockDim.x) {
+        ckey[q] = -1;
+        cval[q] = (T)0;
+    }
     if (threadIdx.x == 0) {
         sh_two_m = 0.0;
         sh_sigma = 0.0;
@@ -964,44 +1037,153 @@ __global__ void k_mod_rows(DevState s, int64_t v0, int64_t v1, const int32_t* la
     __syncthreads();
     const unsigned lane = lane_id();
     const int64_t nloc = v1 - v0;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    double my_two_m = 0.0, my_sigma = 0.0;
-    // labels are given in the caller's vertex order: stored vertex u holds
-    // the label of its original id
-    auto label_of = [&](int64_t u) -> int32_t { return labels[(int64_t)initial_label(s, (int32_t)u) - v0]; };
-    for (int64_t i = warp; i < nloc; i += nwarps) {
-        const int32_t ci = label_of(v0 + i);
-        if (ci < 0 || ci >= nloc) {
-            if (lane == 0) atomicAdd(&acc->bad_label, 1u);
-            continue;
+    const int most_short = width >= 16 ? kModShort : 0;      // few vertices per warp: all lanes on each
+    // Batches from a counter: rows differ by orders of magnitude.  A batch of
+    // 32 takes groups of four vertices from eight places of the range, as hubs
+    // sit next to each other (R-MAT: the ids with few one bits).
+    const int64_t batches = (nloc + width - 1) / width;
+    T my_two_m = (T)0, my_sigma = (T)0;
+    for (;;) {
+        unsigned batch = 0;
+        if (lane == 0) batch = atomicAdd(&acc->next_batch, 1u);
+        batch = __shfl_sync(kFull, batch, 0);
+        if ((int64_t)batch >= batches) break;
+        const int64_t i = width < 32 ? (int64_t)batch * width + lane
+                                     : ((int64_t)(lane >> 2) * batches + batch) * 4 + (lane & 3);
+        bool act = (int)lane < width && i < nloc;
+        int32_t ci = -1;
+        int64_t st = 0, en = 0;
+        if (act) {
+            ci = labels[(int64_t)initial_label(s, (int32_t)(v0 + i)) - v0];
+            st = s.off[v0 + i];
+            en = s.off_end[v0 + i];
+            if (ci < 0 || ci >= nloc) {
+                atomicAdd(&acc->bad_label, 1u);
+                act = false;
+            }
         }
-        double K = 0.0, sg = 0.0;
-        const int64_t st = s.off[v0 + i], en = s.off_end[v0 + i];
-        for (int64_t e = st + lane; e < en; e += 32) {
-            const double w = weight_f64(s, e);
-            K += w;
-            const int64_t j = (int64_t)s.idx[e] - v0;
-            if (j >= 0 && j < nloc && label_of(v0 + j) == ci) sg += w;
+        const int64_t d = act ? en - st : 0;
+        T K = (T)0;
+        bool wide = d > most_short;
+        if (d > kModLong) {
+            const unsigned q = atomicAdd(&acc->long_count, 1u);
+            if (q < (unsigned)kModLongRows) {
+                acc->long_rows[q] = (int32_t)i;
+                wide = false;
+            }
+        } else if (d > 0 && !wide) {
+            mod_walk<1, WK>(s, labels, v0, nloc, st, st, en, ci, vec != 0, 0u, K, my_sigma);
         }
+        __syncwarp();
+        unsigned m = __ballot_sync(kFull, wide);
+        while (m) {
+            const int l = __ffs(m) - 1;
+            m &= m - 1;
+            const int64_t rs = __shfl_sync(kFull, st, l), re = __shfl_sync(kFull, en, l);
+            const int32_t rc = __shfl_sync(kFull, ci, l);
+            T k = (T)0;
+            mod_walk<32, WK>(s, labels, v0, nloc, rs, rs, re, rc, vec != 0, lane, k, my_sigma);
+            __syncwarp();
+            for (int o = 16; o > 0; o >>= 1) k += __shfl_xor_sync(kFull, k, o);
+            if ((int)lane == l) K = k;
+        }
+        my_two_m += K;
+        // the K_i of the batch's first label summed over the warp, then those of
+        // the others one by one, into the block's cache
+        const bool has = K != (T)0;
+        const unsigned hm = __ballot_sync(kFull, has);
+        if (hm == 0u) continue;                             // warp-uniform
+        const int first = __ffs(hm) - 1;
+        const int32_t first_label = __shfl_sync(kFull, ci, first);     // every lane takes part
+        const bool same = has && ci == first_label;
+        T sum = same ? K : (T)0;
+        if (__popc(__ballot_sync(kFull, same)) > 1) {
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
+        }
+        if (has && (!same || (int)lane == first)) {
+            const T add = same ? sum : K;
+            const unsigned slot = ((uint32_t)ci * 0x9E3779B1u) >> 24;
+            const int32_t old = atomicCAS(&ckey[slot], -1, ci);
+            if (old == -1 || old == ci) atomicAdd(&cval[slot], add);
+            else atomicAdd(&Sigma[ci], (double)add);
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        my_two_m += __shfl_xor_sync(kFull, my_two_m, o);
+        my_sigma += __shfl_xor_sync(kFull, my_sigma, o);
+    }
+    if (lane == 0) {
+        atomicAdd(&sh_two_m, (double)my_two_m);
+        atomicAdd(&sh_sigma, (double)my_sigma);
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < kModSlots; q += blockDim.x)
+        if (ckey[q] >= 0) atomicAdd(&Sigma[ckey[q]], (double)cval[q]);
+    if (threadIdx.x == 0) {
+        atomicAdd(&acc->two_m, sh_two_m);
+        atomicAdd(&acc->sigma, sh_sigma);
+    }
+}
+static_assert(kModSlots == 256, "the slot is the top byte of the hash");
+
+// The rows k_mod_rows listed: a block per row, and the rows of more than
+// kModSlice entries in slices over the whole grid.
+template <int WK>
+__global__ void __launch_bounds__(kModThreads) k_mod_long(DevState s, int64_t v0, int64_t v1, const int32_t* labels,
+                                                          double* Sigma, ModAccum* acc, int vec) {
+    __shared__ double sh[2];
+    const int64_t nloc = v1 - v0;
+    const int rows = (int)min(acc->long_count, (unsigned)kModLongRows);
+    if (threadIdx.x < 2) sh[threadIdx.x] = 0.0;
+    __syncthreads();
+    double my_two_m = 0.0, my_sigma = 0.0;               // thread 0: this block's totals
+    // entries [e0, e1) of listed row i, by the whole block
+    auto part = [&](int64_t i, int64_t st, int64_t e0, int64_t e1) {
+        const int32_t ci = labels[(int64_t)initial_label(s, (int32_t)(v0 + i)) - v0];
+        ModSum<WK> K = 0, sg = 0;
+        mod_walk<kModThreads, WK>(s, labels, v0, nloc, e0, st, e1, ci, vec != 0, threadIdx.x, K, sg);
+        __syncwarp();
         for (int o = 16; o > 0; o >>= 1) {
             K += __shfl_xor_sync(kFull, K, o);
             sg += __shfl_xor_sync(kFull, sg, o);
         }
-        if (lane == 0) {
-            atomicAdd(&Sigma[ci], K);
-            my_two_m += K;
-            my_sigma += sg;
+        if (lane_id() == 0) {
+            atomicAdd(&sh[0], (double)K);
+            atomicAdd(&sh[1], (double)sg);
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            atomicAdd(&Sigma[ci], sh[0]);
+            my_two_m += sh[0];
+            my_sigma += sh[1];
+            sh[0] = sh[1] = 0.0;
+        }
+        __syncthreads();
+    };
+    for (int r = blockIdx.x; r < rows; r += gridDim.x) {
+        const int64_t i = acc->long_rows[r];
+        const int64_t st = s.off[v0 + i], en = s.off_end[v0 + i];
+        if (en - st <= kModSlice) part(i, st, st, en);   // block-uniform
+    }
+    for (int base = 0; base < rows; base += kModThreads) {
+        const int r = base + (int)threadIdx.x;
+        bool giant = false;
+        if (r < rows) {
+            const int64_t i = acc->long_rows[r];
+            giant = s.off_end[v0 + i] - s.off[v0 + i] > kModSlice;
+        }
+        if (!__syncthreads_or(giant)) continue;          // block-uniform
+        for (int q = base; q < min(base + kModThreads, rows); ++q) {
+            const int64_t i = acc->long_rows[q];
+            const int64_t st = s.off[v0 + i], en = s.off_end[v0 + i];
+            if (en - st <= kModSlice) continue;          // block-uniform
+            for (int64_t e0 = st + (int64_t)blockIdx.x * kModLong; e0 < en; e0 += (int64_t)gridDim.x * kModLong)
+                part(i, st, e0, min(e0 + kModLong, en));
         }
     }
-    if (lane == 0) {
-        atomicAdd(&sh_two_m, my_two_m);
-        atomicAdd(&sh_sigma, my_sigma);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        atomicAdd(&acc->two_m, sh_two_m);
-        atomicAdd(&acc->sigma, sh_sigma);
+    if (threadIdx.x == 0 && rows > 0) {
+        atomicAdd(&acc->two_m, my_two_m);
+        atomicAdd(&acc->sigma, my_sigma);
     }
 }
 
@@ -1018,12 +1200,34 @@ __global__ void k_mod_null(const double* Sigma, int64_t n, ModAccum* acc) {
     if (threadIdx.x == 0) atomicAdd(&acc->null_sum, sh);
 }
 
-cudaError_t launch_modularity(const DevState& s, int64_t v0, int64_t v1, const int32_t* labels, double* Sigma,
-                              ModAccum* acc, cudaStream_t st, int sms) {
-    k_mod_rows<<<sms * 8, 256, 0, st>>>(s, v0, v1, labels, Sigma, acc);
-    cudaError_t err = cudaGetLastError();
+template <int WK>
+static cudaError_t launch_mod_rows(const DevState& s, int64_t v0, int64_t v1, int64_t max_degree, const int32_t* labels,
+                                   double* Sigma, ModAccum* acc, cudaStream_t st, int sms) {
+    const int64_t nloc = v1 - v0;
+    const int64_t warps = (int64_t)sms * 8 * (kModThreads / 32);     // a full grid's
+    int width = 1;
+    while (width < 32 && width * warps < nloc) width *= 2;
+    const int64_t want = (nloc + (int64_t)width * (kModThreads / 32) - 1) / ((int64_t)width * (kModThreads / 32));
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)sms * 8));
+    const int vec = (reinterpret_cast<uintptr_t>(s.idx) & 15u) == 0 ? 1 : 0;
+    k_mod_rows<WK><<<blocks, kModThreads, 0, st>>>(s, v0, v1, labels, Sigma, acc, width, vec);
+    const cudaError_t err = cudaGetLastError();
+    if (err != cudaSuccess || max_degree <= kModLong) return err;
+    k_mod_long<WK><<<sms * 4, kModThreads, 0, st>>>(s, v0, v1, labels, Sigma, acc, vec);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_modularity(const DevState& s, int64_t v0, int64_t v1, int64_t max_degree, const int32_t* labels,
+                              double* Sigma, ModAccum* acc, cudaStream_t st, int sms) {
+    cudaError_t err;
+    switch (s.weight_kind) {
+        case W_UNIT: err = launch_mod_rows<W_UNIT>(s, v0, v1, max_degree, labels, Sigma, acc, st, sms); break;
+        case W_U32: err = launch_mod_rows<W_U32>(s, v0, v1, max_degree, labels, Sigma, acc, st, sms); break;
+        case W_U8: err = launch_mod_rows<W_U8>(s, v0, v1, max_degree, labels, Sigma, acc, st, sms); break;
+        default: err = launch_mod_rows<W_F32>(s, v0, v1, max_degree, labels, Sigma, acc, st, sms);
+    }
     if (err != cudaSuccess) return err;
-    k_mod_null<<<sms * 4, 256, 0, st>>>(Sigma, v1 - v0, acc);
+    k_mod_null<<<(int)std::min<int64_t>((v1 - v0 + 255) / 256, (int64_t)sms * 4), 256, 0, st>>>(Sigma, v1 - v0, acc);
     return cudaGetLastError();
 }
 

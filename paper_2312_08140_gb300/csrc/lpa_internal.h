@@ -14,6 +14,7 @@
 
 #include <cuda_runtime.h>
 #include <math.h>
+#include <stddef.h>
 #include <stdint.h>
 
 namespace lpa {
@@ -301,14 +302,22 @@ cudaError_t launch_weights_to_u32(float* w, int64_t E, cudaStream_t st, int sms)
 cudaError_t launch_weights_to_u8(const float* w, unsigned char* out, int64_t E, cudaStream_t st, int sms);
 
 // Modularity (Eq. 1), fp64.  Vertex range [v0, v1), labels local to v0.
+constexpr int64_t kModLong = 2048;     // longer rows take a block each,
+constexpr int kModLongRows = 8192;     // up to this many of them
+constexpr int64_t kModSlice = 65536;   // and rows beyond this many entries the whole grid
 struct ModAccum {
     double two_m;
     double sigma;
     double null_sum;
     unsigned int bad_label;
+    unsigned int long_count;            // rows of more than kModLong entries
+    unsigned int next_batch;            // vertices are taken in batches
     unsigned int pad;
+    int32_t long_rows[kModLongRows];    // the first of the long rows (v - v0)
 };
-cudaError_t launch_modularity(const DevState& s, int64_t v0, int64_t v1, const int32_t* labels,
+constexpr size_t kModAccumHead = offsetof(ModAccum, long_rows);   // what the host reads
+// max_degree: of the vertices, or any upper bound.
+cudaError_t launch_modularity(const DevState& s, int64_t v0, int64_t v1, int64_t max_degree, const int32_t* labels,
                               double* Sigma, ModAccum* acc, cudaStream_t st, int sms);
 
 }  // namespace lpa

@@ -37,7 +37,7 @@ namespace {
 
 constexpr int64_t kNoAllocMaxVertices = 1 << 20;
 constexpr size_t kSigmaBytes = (size_t)kNoAllocMaxVertices * sizeof(double);
-constexpr size_t kScratchBytes = kSigmaBytes + 256;   // + ModAccum
+constexpr size_t kScratchBytes = kSigmaBytes + sizeof(ModAccum);
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
@@ -153,10 +153,10 @@ extern "C" lpa_status lpa_modularity_noalloc(int64_t n, int64_t nnz, const int64
     s.w = weights;
 
     cudaError_t e = cudaMemsetAsync(Sigma, 0, (size_t)n * sizeof(double), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(acc, 0, sizeof(ModAccum), st);
-    if (e == cudaSuccess) e = launch_modularity(s, 0, n, labels, Sigma, acc, st, sms);
+    if (e == cudaSuccess) e = cudaMemsetAsync(acc, 0, kModAccumHead, st);
+    if (e == cudaSuccess) e = launch_modularity(s, 0, n, nnz, labels, Sigma, acc, st, sms);
     ModAccum a{};
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&a, acc, sizeof(a), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&a, acc, kModAccumHead, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_err(e);
     if (a.bad_label) return err(LPA_ERR_INVALID_ARG, "labels outside [0, n)");
