@@ -627,7 +627,16 @@ __global__ void __launch_bounds__(kFrontThreads) k_finish(DevState s, int mode, 
             const int64_t v0 = ch * kVertsPerThread;
             uint4 raw = make_uint4(0, 0, 0, 0);
             uint32_t pick = 0;
-            if (ch < nchunks && load_flags(s.flags, s.N, v0, !catch_up, raw)) {
+            if (role == kRoleStartAll) {
+                // marked for whichever compaction comes next; the sweep writes no marks
+                for (int q = 0; q < kVertsPerThread && v0 + q < s.N; ++q) {
+                    const int32_t g = s.gid[v0 + q];
+                    if (g >= 0 && !s.done[g]) {
+                        pick |= 1u << q;
+                        s.flags[v0 + q] = 1;
+                    }
+                }
+            } else if (ch < nchunks && load_flags(s.flags, s.N, v0, !catch_up, raw)) {
                 pick = flag_mask(raw);
                 if (catch_up) {
                     pick &= ~(uint32_t)s.fr_bits[ch];       // scanned this sweep: keep the mark

@@ -219,6 +219,7 @@ enum FinishRole {
     kRoleCatchUp = 1,     // async: compaction of the catch-up set only
     kRoleControl = 2,     // end of a serving cycle: apply, control; marks stay for the next cycle
     kRoleStartSweep = 3,  // start of a serving cycle: compaction (also of newly admitted requests)
+    kRoleStartAll = 4,    // the same, taking every vertex of the requests that are not done
 };
 cudaError_t launch_finish(const DevState& s, int mode, int role, cudaGraphConditionalHandle h, int in_graph,
                           cudaStream_t st, int sms);

@@ -219,6 +219,7 @@ struct Request {
     float* d_w = nullptr;
     bool weighted = false;
     int64_t est_bytes = 0;
+    int64_t max_degree = 0;     // longest row, as the offsets say
 };
 
 }  // namespace
@@ -285,21 +286,34 @@ int grid_for(int64_t n, int sms) {
 
 // One cycle over the arena: compaction, one sweep (two passes in async mode),
 // per-slot control.  Leaves the done flags in S->h_done.
-cudaError_t run_cycle(lpa_server* S) {
+//
+// `entries` and `max_degree` are those of the active requests.  While they hold
+// few entries, a synchronous cycle scans all their vertices: the marks of small
+// graphs collide in a few sectors (40-100 us per sweep, against about 16 us for
+// a dense sweep of 1 M entries).  A bin that no active row reaches is not
+// launched (the three row kernels and the overflow path take about 25 us per
+// cycle just to find their lists empty).
+cudaError_t run_cycle(lpa_server* S, int64_t entries, int64_t max_degree) {
     DevState s = S->s;
     const int mode = S->cfg.mode == LPA_MODE_ASYNC ? MODE_ASYNC : MODE_SYNC;
     cudaGraphConditionalHandle none = 0;
     cudaStream_t st = S->run_st;
     const int passes = mode == MODE_ASYNC ? 2 : 1;
+    const bool all = mode == MODE_SYNC && entries <= kDenseEntries;
+    const int sweep_mode = all ? MODE_SYNC_FULL : mode;              // no marks when every vertex is scanned
+    const int64_t limit[kBins] = {0, s.small_max, s.warp_max, s.mid_max, s.large_max};
+    // only longer rows can overflow the last bin's table
+    s.ovf_possible = 2 * max_degree > kLargeSlots ? 1 : 0;
     cudaError_t e = cudaSuccess;
     for (int p = 0; p < passes && e == cudaSuccess; ++p) {
         // compaction: the cycle's frontier, then (async) the catch-up set
-        e = launch_finish(s, mode, p == 0 ? kRoleStartSweep : kRoleCatchUp, none, 0, st, S->sms);
-        if (e == cudaSuccess) e = launch_sweep_small(s, mode, st, S->sms);
-        if (e == cudaSuccess)
-            e = mode == MODE_ASYNC ? launch_sweep_warp(s, mode, st, S->sms) : launch_sweep_lane(s, mode, st, S->sms);
+        e = launch_finish(s, mode, p == 0 ? (all ? kRoleStartAll : kRoleStartSweep) : kRoleCatchUp, none, 0, st, S->sms);
+        if (e == cudaSuccess) e = launch_sweep_small(s, sweep_mode, st, S->sms);
+        if (e == cudaSuccess && max_degree > limit[1])
+            e = mode == MODE_ASYNC ? launch_sweep_warp(s, mode, st, S->sms)
+                                   : launch_sweep_lane(s, sweep_mode, st, S->sms);
         for (int b = 2; b < kBins && e == cudaSuccess; ++b)
-            e = launch_sweep_block(s, mode, b, S->sms, st);
+            if (max_degree > limit[b]) e = launch_sweep_block(s, sweep_mode, b, S->sms, st);
     }
     if (e == cudaSuccess) e = launch_finish(s, mode, kRoleControl, none, 0, st, S->sms);   // apply + control
     if (e == cudaSuccess) e = cudaMemcpyAsync(S->h_done, s.done, (size_t)S->S * 4, cudaMemcpyDeviceToHost, st);
@@ -397,7 +411,15 @@ void worker_main(lpa_server* S) {
                 S->bad);
             if (e == cudaSuccess) e = cudaGetLastError();
         }
-        if (e == cudaSuccess) e = run_cycle(S);
+        int64_t entries = 0, max_degree = 0;
+        {
+            std::lock_guard<std::mutex> lock(S->mu);
+            for (auto& kv : S->active) {
+                entries += kv.second->nnz;
+                max_degree = std::max(max_degree, kv.second->max_degree);
+            }
+        }
+        if (e == cudaSuccess) e = run_cycle(S, entries, max_degree);
         S->cycles++;
         if (e != cudaSuccess) {
             std::lock_guard<std::mutex> lock(S->mu);
@@ -608,6 +630,8 @@ lpa_status lpa_serve_submit(lpa_server_t S, int64_t n, int64_t nnz, const int64_
     r->n = n;
     r->nnz = nnz;
     r->weighted = weights != nullptr;
+    for (int64_t i = 0; i < n; ++i) 
+        r->max_degree = std::max(r->max_degree, (int64_t)((uint64_t)offsets[i + 1] - (uint64_t)offsets[i]));
     if (n == 0 || solo) {
         std::lock_guard<std::mutex> lock(S->mu);
         if (solo) {
