@@ -161,7 +161,10 @@ typedef struct {
 
 /* Launch parameters of the sweep.  Vertices are binned by degree d:
  *   d <= small_max                  one thread per vertex, row held in registers
- *   small_max < d <= warp_max       one warp per vertex, per-warp shared-memory table
+ *   small_max < d <= warp_max       asynchronous: one warp per vertex, per-warp
+ *                                   shared-memory table; synchronous: one lane per
+ *                                   vertex, its row sorted in registers (rows of more
+ *                                   than 64 entries: one warp)
  *   warp_max  < d <= mid_max        one 128-thread block per vertex, shared table
  *   mid_max   < d <= large_max      one 256-thread block per vertex, shared table
  *   d > large_max                   one 512-thread block per vertex, 8192-slot shared
@@ -173,7 +176,10 @@ typedef struct {
  *                                   block per partition)
  * A sweep is "dense" (every vertex with an entry is scanned, no frontier
  * compaction) when the vertices changed since the previous compaction hold
- * at least dense_permille / 1000 of all entries; the first sweep is always
+ * at least dense_permille / 1000 of all entries (a synchronous sweep that did
+ * so also lets the next one write no marks, which makes the one after it dense
+ * too, and a synchronous run of at most 4 M entries is dense throughout, both
+ * unless dense_permille is 1001); the first sweep is always
  * dense (Algorithm 1 starts with every vertex unprocessed); 1001 = never
  * otherwise.  Scanning a vertex whose neighbours did not change never
  * changes its label in LPA_MODE_SYNC, so this choice affects speed only.

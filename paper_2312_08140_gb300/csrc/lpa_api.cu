@@ -243,13 +243,13 @@ lpa_status setup_blocks(Engine& E, cudaStream_t st) {
     if (E.s.G == 1 && block_entries >= (unsigned long long)kMajorityEntries) {
         void* m[2] = {nullptr, nullptr};
         const size_t mb[2] = {((size_t)E.s.N / 32 + 1) * sizeof(uint32_t), (size_t)E.s.N * sizeof(int32_t)};
-        for (int k = 0; k < 2; ++k) {
-            if (pool_alloc(E.device, &m[k], mb[k]) != cudaSuccess) {
-                cudaGetLastError();
-                return fail(LPA_ERR_OUT_OF_MEMORY, "majority scratch: %zu bytes", mb[k]);
-            }
-            E.dom_scratch.push_back(m[k]);
+        if (pool_alloc(E.device, &m[0], mb[0]) != cudaSuccess || pool_alloc(E.device, &m[1], mb[1]) != cudaSuccess) {
+            // no room: the ordinary kernels take every row
+            cudaGetLastError();
+            if (m[0]) E.dom_scratch.push_back(m[0]);
+            return LPA_OK;
         }
+        E.dom_scratch.assign(m, m + 2);
         E.s.dom_bits = static_cast<uint32_t*>(m[0]);
         E.s.defer = static_cast<int32_t*>(m[1]);
     }

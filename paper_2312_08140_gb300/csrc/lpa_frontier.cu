@@ -19,7 +19,9 @@ namespace lpa {
 
 constexpr int kFrontThreads = 256;
 constexpr int kVertsPerThread = 16;
-constexpr int kFinishVerts = 2048;      // vertices per block of k_finish, up to a full chip
+constexpr int kFinishVerts = 2048;      // vertices per block of k_finish, up to a full chip: half of the
+                                        // 4096 that its compaction step takes at a time, so that the
+                                        // change lists of a sparse sweep spread over enough blocks
 
 __global__ void k_set_params(Ctrl* ctrl, double tau, int max_iters, int mode, int nonstrict, int prune_other,
                              int32_t* labels_out, int local_ids) {
@@ -413,9 +415,9 @@ __device__ __forceinline__ long long warp_sum(long long x) {
 //
 // Nothing else runs meanwhile, so its time is the latency of its loads: lane b
 // of the first warp owns bin b, every counter it needs is loaded at once, and
-// the totals are warp sums.  (One thread reading and writing the counters of
-// the five bins in turn took 12 of the 15 us that k_finish spent on a
-// 10,000-vertex graph.)
+// the totals are warp sums (k_finish of a dense sweep: 14-18 us when one
+// thread read and wrote the counters of the five bins in turn, 8 us now on a
+// 10,000-vertex graph and 10 us on 16.8 M vertices).
 __device__ void control_step(const DevState& s, int mode, int role, int dense_next, cudaGraphConditionalHandle h,
                              int in_graph) {
     Ctrl* c = s.ctrl;
@@ -525,7 +527,12 @@ __device__ void control_step(const DevState& s, int mode, int role, int dense_ne
             bool skip = high && last_high;
             // Synchronous labels do not depend on the frontier, so there a mark
             // is only worth its store (and the sparse sweep its compaction) when
-            // the next frontier will be small.
+            // the next frontier will be small.  A mark costs about as much as a
+            // gather (batch of 256 graphs: 550 us for 81 M), and the frontier
+            // after a sweep that changed half of the entries is nearly all
+            // vertices.  Skipping from 3/10 on would cost more than it saves
+            // there: the sweep after next then scans 219 M entries in 1.6 ms
+            // instead of 92 M in 0.7.
             if (mode != MODE_ASYNC && s.dense_permille <= 1000)
                 skip = skip || s.active_entries <= kDenseEntries ||
                        changed * 1000.0 >= (double)s.dense_permille * active;
@@ -1023,7 +1030,7 @@ __device__ __forceinline__ void mod_walk(const DevState& s, const int32_t* label
 // matters, so the warp first adds up the K_i that share the batch's first label,
 // and the block keeps sums in a small shared cache: adding every K_i to Sigma by itself serialised on
 // the hot communities (2 M vertices of an R-MAT graph, nearly all in one
-// community: 7.5 ms).
+// community: 7.5 ms, now 0.68; its 60 M gathers take 0.2 ms from L2).
 constexpr int kModThreads = 256;
 constexpr int kModSlots = 256;          // labels cached per block
 constexpr int kModShort = 64;           // longest row a lane takes
