@@ -22,10 +22,11 @@
 //     aggregation steps;
 //   * in step k every thread reads its P ids of tile k+1 from shared memory
 //     and issues their label gathers into registers, then aggregates tile k
-//     (whose labels arrived during step k-1): lanes holding the same label
-//     are grouped with __match_any_sync and the group leader adds the group's
-//     weight into a shared-memory open-addressing table, listing the slots it
-//     fills;
+//     (whose labels arrived during step k-1) into a shared-memory
+//     open-addressing table, listing the slots it fills: unit weights by
+//     groups of lanes that hold the same label (__match_any_sync; the group's
+//     size is its sum), other weights lane by lane (summing each group's
+//     weights took an R-MAT graph with weights 1..1000 30 ms, this 8.9);
 //   * after a row's last tile each warp scans the slots it listed and
 //     reduces (sum, tie key) to its candidate, a shared 64-bit maximum gives
 //     the block's winner, which is recorded, and the neighbours are marked.
@@ -189,10 +190,12 @@ struct RowsShape {
 // thread follow from it).  Measured on R-MAT 27: one 512-thread block per SM
 // for the last bin and two 256-thread blocks for the bin before it ran the
 // run in 107 ms; two and four blocks (64 registers, 4 gathers per thread)
-// took 154 ms, and with 8 gathers per thread (spilling) 136 ms.
-template <int NT>
+// took 154 ms, and with 8 gathers per thread (spilling) 136 ms.  The weighted
+// kernels keep 4 gathers per thread either way and take twice the blocks
+// (R-MAT of 769,230 vertices, weights 1..1000: 8.9 -> 8.3 ms).
+template <int NT, int WK>
 struct RowsOccupancy {
-    static constexpr int kBlocks = NT >= 512 ? 1 : NT >= 256 ? 2 : 8;
+    static constexpr int kBlocks = (NT >= 512 ? 1 : NT >= 256 ? 2 : 8) * (WK != W_UNIT && NT >= 256 ? 2 : 1);
 };
 
 // Metadata of one row of the current batch.
@@ -214,7 +217,7 @@ struct ProdState {
 };
 
 template <bool ASYNC, int WK, bool BATCH, bool NS, int NT>
-__global__ void __launch_bounds__(NT, RowsOccupancy<NT>::kBlocks) k_sweep_rows(DevState s, int bin,
+__global__ void __launch_bounds__(NT, RowsOccupancy<NT, WK>::kBlocks) k_sweep_rows(DevState s, int bin,
                                                                             int flag_neighbours) {
     using T = typename Acc<WK>::T;
     using Sh = RowsShape<NT, WK>;
@@ -652,13 +655,11 @@ __global__ void __launch_bounds__(NT, RowsOccupancy<NT>::kBlocks) k_sweep_rows(D
                     const bool ok = lab_cur[p] != kEmptyKey;
                     T wsum = w_cur[p];
                     bool lead = ok;
-                    if constexpr (WK != W_F32) {
+                    // weights go in lane by lane: summing them per group costs
+                    // 129 cycles of an SM for 32 distinct labels
+                    if constexpr (WK == W_UNIT) {
                         const unsigned peers = __match_any_sync(kFull, lab_cur[p]);
-                        if constexpr (WK == W_UNIT) {
-                            wsum = (T)__popc(peers);
-                        } else {
-                            wsum = __reduce_add_sync(peers, wsum);
-                        }
+                        wsum = (T)__popc(peers);
                         lead = ok && lane == (unsigned)(__ffs(peers) - 1);
                     }
                     list_created(lead ? insert(lab_cur[p], wsum) : -1);

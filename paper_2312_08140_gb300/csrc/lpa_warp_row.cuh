@@ -1,6 +1,8 @@
-// lpa_warp_row.cuh -- a whole warp on one row: the label sums of a row of more
-// than 32 entries in a per-warp open-addressing table in shared memory.
-// Shared by the asynchronous warp kernel and the synchronous lane kernel.
+// lpa_warp_row.cuh -- a whole warp (or block) on one row: 16-byte reads of a
+// row's ids and its neighbours' marks (row and majority kernels), per-label
+// sums by lane groups and a per-warp open-addressing table in shared memory
+// (warp kernel), and the label sums of a row of more than 32 entries (lane
+// kernel, for the rows it does not sort).
 #pragma once
 
 #include "lpa_device.cuh"
