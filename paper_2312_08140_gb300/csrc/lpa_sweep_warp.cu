@@ -38,7 +38,12 @@ constexpr unsigned kAsyncMaxRunBatches = 8;   // async: batches a warp walks in 
 constexpr unsigned kAsyncSmallRunBatches = 2;  // async, a bin of one wave of batches: batches per run
 constexpr unsigned kScatterWindow = 4096;   // batches per scattered window (a power of two)
 
-template <int WK, bool BATCH, bool NS>
+// DOM: the graph has majority kernels, so a pass may scan only the rows they
+// left over and clears the bits of vertices that leave the dominating label.
+// Batches and smaller graphs have none and are compiled without the two tests:
+// the first sweep of an asynchronous batch (256 planted partitions, 58 M
+// entries, unit weights) takes 1180 us, 1270 with them.
+template <int WK, bool BATCH, bool NS, bool DOM>
 __global__ void __launch_bounds__(kWarpThreads, 4) k_sweep_warp(DevState s, int flag_neighbours) {
     using T = typename Acc<WK>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -59,8 +64,12 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_sweep_warp(DevState s, int 
     }
     __syncwarp();
 
-    const BinView bv = bin_view(s, 1);
-    const Labels L = labels_of(s);
+    BinView bv = bin_view(s, 1);
+    Labels L = labels_of(s);
+    if constexpr (!DOM) {
+        bv.left = nullptr;
+        L.dom_bits = nullptr;
+    }
     const bool marks = marks_on(s, flag_neighbours);
     const uint32_t sweep = NS ? (uint32_t)s.ctrl->iter + 1u : 0u;   // non-strict tie-break (Section 4.1.5)
     const bool po = s.ctrl->prune_other != 0;               // FLPA's pruning rule
@@ -369,10 +378,10 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_sweep_warp(DevState s, int 
     flush_bin_counts(s, 1, my_changed, my_changed_entries);
 }
 
-template <int WK, bool BATCH, bool NS>
-static cudaError_t launch_warp_t(const DevState& s, int flag, cudaStream_t st, int sms) {
+template <int WK, bool BATCH, bool NS, bool DOM>
+static cudaError_t launch_warp_k(const DevState& s, int flag, cudaStream_t st, int sms) {
     const size_t smem = (size_t)kWarpsPerBlock * s.warp_slots * 9;     // table + list of filled slots
-    auto kern = k_sweep_warp<WK, BATCH, NS>;
+    auto kern = k_sweep_warp<WK, BATCH, NS, DOM>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     int per_sm = 0;
@@ -381,6 +390,14 @@ static cudaError_t launch_warp_t(const DevState& s, int flag, cudaStream_t st, i
     if (per_sm < 1) per_sm = 1;
     kern<<<sms * per_sm, kWarpThreads, smem, st>>>(s, flag);
     return cudaGetLastError();
+}
+
+template <int WK, bool BATCH, bool NS>
+static cudaError_t launch_warp_t(const DevState& s, int flag, cudaStream_t st, int sms) {
+    if constexpr (!BATCH) {
+        if (s.dom_bits) return launch_warp_k<WK, BATCH, NS, true>(s, flag, st, sms);
+    }
+    return launch_warp_k<WK, BATCH, NS, false>(s, flag, st, sms);
 }
 
 template <bool BATCH, bool NS>
