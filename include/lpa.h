@@ -177,10 +177,10 @@ typedef struct {
  * A sweep is "dense" (every vertex with an entry is scanned, no frontier
  * compaction) when the vertices changed since the previous compaction hold
  * at least dense_permille / 1000 of all entries (a synchronous sweep that did
- * so also lets the next one write no marks, which makes the one after it dense
- * too, and a synchronous run of at most 4 M entries is dense throughout, both
- * unless dense_permille is 1001); the first sweep is always
- * dense (Algorithm 1 starts with every vertex unprocessed); 1001 = never
+ * so -- on graphs of at most 4 M entries, one that changed vertices of at least
+ * 1 / 1000 of them -- also lets the next one write no marks, which makes the one
+ * after it dense too, both unless dense_permille is 1001); the first sweep is
+ * always dense (Algorithm 1 starts with every vertex unprocessed); 1001 = never
  * otherwise.  Scanning a vertex whose neighbours did not change never
  * changes its label in LPA_MODE_SYNC, so this choice affects speed only.
  * lpa_graph_set_config validates: 1 <= small_max <= 8, small_max < warp_max

@@ -533,9 +533,12 @@ __device__ void control_step(const DevState& s, int mode, int role, int dense_ne
             // vertices.  Skipping from 3/10 on would cost more than it saves
             // there: the sweep after next then scans 219 M entries in 1.6 ms
             // instead of 92 M in 0.7.
-            if (mode != MODE_ASYNC && s.dense_permille <= 1000)
-                skip = skip || s.active_entries <= kDenseEntries ||
-                       changed * 1000.0 >= (double)s.dense_permille * active;
+            // Graphs of at most kDenseEntries entries stay dense much longer.
+            if (mode != MODE_ASYNC && s.dense_permille <= 1000) {
+                const int from = s.active_entries <= kDenseEntries ? min(kDensePermille, s.dense_permille)
+                                                                   : s.dense_permille;
+                skip = skip || changed * 1000.0 >= (double)from * active;
+            }
             c->skip_marks = skip && allow_dense ? 1 : 0;
             c->last_pass_high = high ? 1 : 0;
             c->pass_changed_entries = 0;

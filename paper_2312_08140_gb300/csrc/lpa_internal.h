@@ -24,12 +24,18 @@ constexpr int kBins = 5;                // thread / warp / 128-, 256-, 512-threa
 constexpr int kBlockBins = 3;           // bins 2..4 use the block kernel
 constexpr int kBlockThreads[kBlockBins] = {128, 256, 512};
 constexpr int kHighPermille = 900;      // "almost every vertex changed" (see skip_marks)
-// Synchronous runs of graphs up to this many entries scan every vertex in
-// every sweep.  The byte marks of a small graph collide in a few 32-byte
-// sectors: 10,000 vertices, 160 K entries: 40-100 us per sweep with marks, 10
-// without; 40,000 vertices, 0.9 M entries: 50-115 us against 16.  At 4 M
-// entries a dense sweep takes about 30 us.
+// Synchronous runs of graphs up to kDenseEntries entries scan every vertex in
+// the next sweep, without marks, while a sweep changes vertices of at least
+// kDensePermille / 1000 of the entries.  The byte marks of a small graph
+// collide in a few 32-byte sectors: 10,000 vertices, 160 K entries: 40-100 us
+// per sweep with marks, 24 without, as long as some percent of the entries
+// change; 130,000 vertices, 3.9 M entries: 71 us against 37 at 2.4%, 55 against
+// 47 (with the finish kernel) at 0.3%.  Below a thousandth the marks cost
+// nothing and a frontier of a few rows is the cheaper sweep: R-MAT of 131,072
+// vertices and 3.7 M entries, a limit cycle of 60-odd vertices: 100 sweeps take
+// 10.2 ms dense throughout, 4.6 with this line.
 constexpr long long kDenseEntries = 4 << 20;
+constexpr int kDensePermille = 1;
 constexpr int kSliceLen = 4096;         // entries per slice of an overflowing row
 constexpr int kMaxParts = 4096;         // partitions a row may use on the sliced path
 constexpr int kMaxSlices = 4096;        // slices a row may use on the sliced path (with the above: d <= 2^24)
