@@ -542,6 +542,8 @@ __device__ void control_step(const DevState& s, int mode, int role, int dense_ne
             c->skip_marks = skip && allow_dense ? 1 : 0;
             c->last_pass_high = high ? 1 : 0;
             c->pass_changed_entries = 0;
+            // a serving cycle's host side takes it with the done flags
+            if (role == kRoleControl) s.done[s.G] = (int32_t)min(pass_changed, 0x7fffffffull);
         }
     } else if (bin) {
         c->sweep_bin_vertices[b] = swv;

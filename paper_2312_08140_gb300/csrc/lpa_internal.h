@@ -174,7 +174,7 @@ struct DevState {
     int64_t active_entries;    // entries of all vertices with an entry (= E)
     Ctrl* ctrl;
     unsigned long long* dN;    // [G] changed vertices of the current sweep
-    int32_t* done;             // [G]
+    int32_t* done;             // [G] (serving: one more word, see control_step)
     int32_t* iters;            // [G]
     int32_t* exit_reason;      // [G]
     long long* hist_changed;   // [G * kMaxHist]

@@ -53,3 +53,36 @@ def test_small_graph_takes_frontiers_in_a_long_tail(cycle):
     # scans the neighbours of the vertices that changed
     assert info["scanned"][5:] == [front for _, _, front in trace[4:-1]]
     assert info["scanned"][1] == info["scanned"][2] == g.nnz
+
+
+@pytest.mark.gpu
+def test_serving_through_a_tail_and_back(cycle):
+    """A request in its tail (frontiers) is joined by others (every vertex again):
+    each result is the oracle's."""
+    import time
+
+    import paper_2312_08140_gb300 as lpa
+    g, trace, _ = cycle
+    cap = 60
+    others = [L.planted_partition(3000, 6, seed=2), L.rmat(12, 16, seed=9)]
+    srv = lpa.lpa_serve_create(1 << 30, 1 << 18, 1 << 23, 8, "sync", 0.0, cap)
+    try:
+        todo = {lpa.lpa_serve_submit(srv, g.n, g.nnz, g.off, g.idx, g.w): g}
+        for q in others:
+            before = lpa.lpa_serve_stats(srv)["cycles"]
+            t0 = time.time()
+            while lpa.lpa_serve_stats(srv)["cycles"] < before + 12 and time.time() - t0 < 0.02:
+                time.sleep(0.0002)
+            todo[lpa.lpa_serve_submit(srv, q.n, q.nnz, q.off, q.idx, q.w)] = q
+        done, t0 = set(), time.time()
+        while len(done) < len(todo):
+            done.update(lpa.lpa_serve_poll(srv))
+            assert time.time() - t0 < 60, "serving did not finish"
+            time.sleep(0.0005)
+        for ticket, q in todo.items():
+            labels, info = lpa.lpa_serve_fetch(srv, ticket, q.n)
+            ref, it, changed = O.lpa_sync(q.off, q.idx, q.w, 0.0, cap)
+            assert info.iterations == it and list(info.changed[:it]) == changed.tolist()[:it]
+            assert np.array_equal(labels, ref)
+    finally:
+        lpa.lpa_serve_destroy(srv)
