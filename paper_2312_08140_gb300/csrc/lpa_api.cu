@@ -571,12 +571,21 @@ lpa_status engine_view(Engine& E, const Engine& par, int32_t K, const lpa_config
     return LPA_OK;
 }
 
-// `main`: the sweep's main pass, which the majority kernels precede (an
-// asynchronous catch-up pass is small).
+// What precedes the bins of a sweep's main pass (an asynchronous catch-up pass
+// is small): the search for a dominating label and, in the synchronous modes,
+// the rows that it settles.
+cudaError_t launch_pass_start(Engine& E, int mode, cudaStream_t st) {
+    if (!E.s.dom_bits) return cudaSuccess;
+    cudaError_t err = launch_dominant(E.s, 0, st, E.sms);
+    if (err == cudaSuccess && (mode & ~kModeNonstrict) != MODE_ASYNC) err = launch_majority(E.s, mode, 0, st, E.sms);
+    return err;
+}
+
+// `main`: the sweep's main pass.
 cudaError_t launch_bin(Engine& E, int mode, int bin, bool main, cudaStream_t st) {
-    if (main && E.s.dom_bits && bin >= 1) {
+    if (main && E.s.dom_bits && bin >= 1 && (mode & ~kModeNonstrict) == MODE_ASYNC) {
         cudaError_t err = cudaSuccess;
-        if ((mode & ~kModeNonstrict) == MODE_ASYNC && (bin == 2 || bin == 3)) err = launch_dominant(E.s, bin, st, E.sms);
+        if (bin == 2 || bin == 3) err = launch_dominant(E.s, bin, st, E.sms);
         if (err == cudaSuccess) err = launch_majority(E.s, mode, bin, st, E.sms);
         if (err != cudaSuccess) return err;
     }
@@ -601,8 +610,8 @@ int bin_at(int mode, int k) {
 }
 
 cudaError_t enqueue_pass(Engine& E, int mode, bool main, cudaStream_t st) {
-    if (main && E.s.dom_bits) {
-        const cudaError_t err = launch_dominant(E.s, 0, st, E.sms);
+    if (main) {
+        const cudaError_t err = launch_pass_start(E, mode, st);
         if (err != cudaSuccess) return err;
     }
     for (int k = 0; k < kBins; ++k) {
@@ -820,7 +829,7 @@ lpa_status engine_run_profiled(Engine& E, int mode, double tol, int32_t max_iter
         float sweep_ms[kBins] = {0.f}, fin_ms = 0.f;
         const int passes = mode == MODE_ASYNC ? 2 : 1;
         for (int p = 0; p < passes; ++p) {
-            if (p == 0 && E.s.dom_bits) LPA_P(launch_dominant(E.s, 0, st, E.sms));
+            if (p == 0) LPA_P(launch_pass_start(E, mode | (ns ? kModeNonstrict : 0), st));
             for (int k = 0; k < kBins; ++k) {
                 const int b = bin_at(mode, k);
                 LPA_P(cudaEventRecord(ev[k], st));

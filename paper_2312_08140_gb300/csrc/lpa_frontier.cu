@@ -504,11 +504,13 @@ __device__ void control_step(const DevState& s, int mode, int role, int dense_ne
             int per_pass = 1;
             for (int q = 0; q < kBins; ++q) per_pass += s.bin_static[q] ? 1 : 0;
             if (s.bin_static[kBins - 1] && s.ovf_possible) per_pass += 4;   // plan, slices, partitions, rescan
-            int majority = 0;               // once per sweep: sample, bits, one kernel per bin
+            int majority = 0;               // once per sweep: sample, bits, rows (asynchronous: per bin)
             if (s.dom_bits) {
-                majority = 2;
-                for (int q = 1; q < kBins; ++q) majority += s.bin_static[q] ? 1 : 0;
-                if (mode == MODE_ASYNC) majority += (s.bin_static[2] ? 2 : 0) + (s.bin_static[3] ? 2 : 0);
+                majority = 3;
+                if (mode == MODE_ASYNC) {
+                    majority = 2 + (s.bin_static[2] ? 2 : 0) + (s.bin_static[3] ? 2 : 0);
+                    for (int q = 1; q < kBins; ++q) majority += s.bin_static[q] ? 1 : 0;
+                }
             }
             atomicAdd((unsigned long long*)&c->total_sweeps, 1ull);
             atomicAdd((unsigned long long*)&c->total_scanned, (unsigned long long)scn);

@@ -243,10 +243,12 @@ cudaError_t launch_sweep_warp(const DevState& s, int mode, cudaStream_t st, int 
 cudaError_t launch_sweep_lane(const DevState& s, int mode, cudaStream_t st, int sms);
 // Majority kernels (lpa_sweep_majority.cu), for single graphs whose block bins
 // hold kMajorityEntries: launch_dominant looks for a label that dominates the
-// pass and marks its vertices; launch_majority then settles the rows of one bin
-// (1..4) that it decides and leaves the others to the bin's ordinary kernel.
-// When no label dominates, its six to ten launches cost about 20 us a sweep;
-// 4 M entries in the block bins take at least 40 us to gather.
+// pass and marks its vertices; launch_majority then settles the rows that it
+// decides -- of one bin (1..4) in the asynchronous mode, of all bins otherwise --
+// and leaves the others to the bins' ordinary kernels.
+// When no label dominates, their launches (three, asynchronously six to ten)
+// cost about 10 to 20 us a sweep; 4 M entries take at least 40 us to gather.  So
+// sweeps whose frontier holds fewer are not searched either.
 constexpr long long kMajorityEntries = 4 << 20;
 // before_bin 0: at the start of a pass (any sweep but the first); 2, 3: before
 // that bin of an asynchronous pass (the first sweep only).

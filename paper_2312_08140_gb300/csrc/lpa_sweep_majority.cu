@@ -23,6 +23,15 @@
 //                 The row is then settled; other rows are listed and left to the
 //                 bin's ordinary kernel.
 //
+// A frontier of fewer than kMajorityEntries entries (lpa_internal.h) is left to
+// the ordinary kernels without a search.  A synchronous sweep takes the rows of
+// all bins in one launch, where a block that runs out of rows of one bin goes on
+// with the next; an asynchronous pass takes each bin before its ordinary kernel,
+// as rows of one bin may read the new labels of the bins before.  R-MAT 22,
+// synchronous: 1358 -> 1134 us a run by that; a long tail (R-MAT 20, edge factor
+// 8, tolerance 0, 100 sweeps) 8.6 -> 5.4 ms (6.6 without majority kernels, by the
+// ordinary kernels of the time).
+//
 // Measured on R-MAT 26 (1.84 G entries, asynchronous): the three row bins of the
 // second and third sweep 20.5 -> 5.4 ms, the warp bin there 4.3 -> 0.95, the 128-
 // and 256-thread bins of the first sweep 9.7 -> 3.5.
@@ -39,7 +48,6 @@ namespace lpa {
 constexpr int kPickThreads = 1024;
 constexpr int kPickSamples = 4;             // per thread
 constexpr int kMajThreads = 256;
-constexpr int kMajLongThreads = 256;        // last bin: a block per row
 constexpr int kMajVec = 2;                  // 4-entry vectors per lane and step
 
 // `mid`: between two bins of the first asynchronous sweep, where the bins before
@@ -49,6 +57,11 @@ __global__ void __launch_bounds__(kPickThreads) k_dom_pick(DevState s, int mid, 
     __shared__ int ones[31], same;
     Ctrl* c = s.ctrl;
     if ((c->iter == 0) != (mid != 0)) return;
+    // a frontier of a few rows is not worth the search (the label stays off)
+    unsigned long long entries = 0;
+#pragma unroll
+    for (int b = 1; b < kBins; ++b) entries += c->bin_entries[c->rd][b];
+    if (entries < (unsigned long long)kMajorityEntries) return;
     if (threadIdx.x < 31) ones[threadIdx.x] = 0;
     if (threadIdx.x == 31) same = 0;
     __syncthreads();
@@ -218,10 +231,9 @@ __device__ __forceinline__ void leave_rows(const DevState& s, int bin, bool left
 
 // Bin 1: a thread per row, 8 entries at a time.
 template <bool ASYNC, int WK>
-__global__ void __launch_bounds__(kMajThreads) k_majority_lane(DevState s, int flag_neighbours) {
+__device__ __forceinline__ void majority_lane(const DevState& s, int flag_neighbours) {
     using T = typename Acc<WK>::T;
-    Ctrl* c = s.ctrl;
-    if (!c->dom_on) return;
+    const Ctrl* c = s.ctrl;
     const int rd = c->rd;
     const Labels L = labels_of(s);
     const int32_t* list = (L.dense ? s.slist : s.flist) + s.bin_base[1];
@@ -271,10 +283,9 @@ __global__ void __launch_bounds__(kMajThreads) k_majority_lane(DevState s, int f
 
 // Bins 2 and 3: a warp per row, 32 rows taken at a time.
 template <bool ASYNC, int WK>
-__global__ void __launch_bounds__(kMajThreads) k_majority_rows(DevState s, int bin, int flag_neighbours) {
+__device__ __forceinline__ void majority_rows(const DevState& s, int bin, int flag_neighbours) {
     using T = typename Acc<WK>::T;
     Ctrl* c = s.ctrl;
-    if (!c->dom_on) return;
     const int rd = c->rd;
     const Labels L = labels_of(s);
     const int32_t* list = (L.dense ? s.slist : s.flist) + s.bin_base[bin];
@@ -342,13 +353,12 @@ __global__ void __launch_bounds__(kMajThreads) k_majority_rows(DevState s, int b
 // of step t + 1 was last read before the barrier of step t - 1 and is cleared
 // during step t.
 template <bool ASYNC, int WK>
-__global__ void __launch_bounds__(kMajLongThreads) k_majority_block(DevState s, int bin, int flag_neighbours) {
+__device__ __forceinline__ void majority_block(const DevState& s, int bin, int flag_neighbours) {
     using T = typename Acc<WK>::T;
     using A = typename MajSum<WK>::A;
     __shared__ A acc[3][2];
     __shared__ unsigned next_row;
     Ctrl* c = s.ctrl;
-    if (!c->dom_on) return;
     const int rd = c->rd;
     const Labels L = labels_of(s);
     const int32_t* list = (L.dense ? s.slist : s.flist) + s.bin_base[bin];
@@ -371,9 +381,9 @@ __global__ void __launch_bounds__(kMajLongThreads) k_majority_block(DevState s, 
         const int32_t own = ASYNC ? __ldcg(L.C + v) : L.C[v];
         MajSum<WK> m{};
         bool ok = false;
-        for (int64_t e = st & ~(int64_t)3; e < en; e += (int64_t)4 * kMajLongThreads * kMajVec, ++t) {
+        for (int64_t e = st & ~(int64_t)3; e < en; e += (int64_t)4 * kMajThreads * kMajVec, ++t) {
             T in = (T)0, out = (T)0;
-            count_step<WK, kMajLongThreads>(s, e, st, en, v, threadIdx.x, in, out);
+            count_step<WK, kMajThreads>(s, e, st, en, v, threadIdx.x, in, out);
             in = warp_add<WK>(in);
             out = warp_add<WK>(out);
             if (lane == 0) {
@@ -384,7 +394,7 @@ __global__ void __launch_bounds__(kMajLongThreads) k_majority_block(DevState s, 
             __syncthreads();
             m.in += acc[t % 3][0];
             m.out += acc[t % 3][1];
-            const int64_t rest = max((int64_t)0, en - (e + (int64_t)4 * kMajLongThreads * kMajVec));
+            const int64_t rest = max((int64_t)0, en - (e + (int64_t)4 * kMajThreads * kMajVec));
             ok = settled<WK>(s, m, rest, en - st);      // block-uniform
             if (ok || hopeless<WK>(s, m, rest)) {
                 ++t;
@@ -400,13 +410,44 @@ __global__ void __launch_bounds__(kMajLongThreads) k_majority_block(DevState s, 
                     my_changed_entries += (unsigned long long)(en - st);
                 }
             }
-            if (changed && marks) mark_row<ASYNC, kMajLongThreads, 2>(s, L, st, en, v, threadIdx.x, po, label);
+            if (changed && marks) mark_row<ASYNC, kMajThreads, 2>(s, L, st, en, v, threadIdx.x, po, label);
         } else if (threadIdx.x == 0) {
             s.defer[s.bin_base[bin] + atomicAdd(&c->defer_cnt[bin], 1u)] = (int32_t)k;
         }
         __syncthreads();                                // next_row was read
     }
     flush_bin_counts(s, bin, my_changed, my_changed_entries);
+}
+
+// Asynchronous passes: one bin, before its ordinary kernel.  (`flag` is always 1;
+// as a constant it cost k_majority_block 7% on R-MAT 26, 1640 -> 1755 us.)
+template <int WK>
+__global__ void __launch_bounds__(kMajThreads) k_majority_lane(DevState s, int flag) {
+    if (!s.ctrl->dom_on) return;
+    majority_lane<true, WK>(s, flag);
+}
+template <int WK>
+__global__ void __launch_bounds__(kMajThreads) k_majority_rows(DevState s, int bin, int flag) {
+    if (!s.ctrl->dom_on) return;
+    majority_rows<true, WK>(s, bin, flag);
+}
+template <int WK>
+__global__ void __launch_bounds__(kMajThreads) k_majority_block(DevState s, int bin, int flag) {
+    if (!s.ctrl->dom_on) return;
+    majority_block<true, WK>(s, bin, flag);
+}
+
+// Synchronous sweeps: every bin, as no row's pick depends on another's.
+template <int WK>
+__global__ void __launch_bounds__(kMajThreads) k_majority_all(DevState s, int flag_neighbours) {
+    if (!s.ctrl->dom_on) return;
+    majority_block<false, WK>(s, kBins - 1, flag_neighbours);
+    for (int bin = kBins - 2; bin > 1; --bin) {
+        __syncthreads();                                // flush_bin_counts' sums were read
+        majority_rows<false, WK>(s, bin, flag_neighbours);
+    }
+    __syncthreads();
+    majority_lane<false, WK>(s, flag_neighbours);
 }
 
 template <typename K>
@@ -417,38 +458,34 @@ static cudaError_t wave_of(K kern, int threads, int sms, int* blocks) {
     return err;
 }
 
-template <bool ASYNC, int WK>
-static cudaError_t launch_majority_t(const DevState& s, int bin, int flag, cudaStream_t st, int sms) {
+template <int WK>
+static cudaError_t launch_majority_w(const DevState& s, int mode, int bin, cudaStream_t st, int sms) {
     int blocks = 0;
     cudaError_t err;
-    if (bin == 1) {
-        if ((err = wave_of(k_majority_lane<ASYNC, WK>, kMajThreads, sms, &blocks)) != cudaSuccess) return err;
-        k_majority_lane<ASYNC, WK><<<blocks, kMajThreads, 0, st>>>(s, flag);
-    } else if (bin < kBins - 1) {
-        if ((err = wave_of(k_majority_rows<ASYNC, WK>, kMajThreads, sms, &blocks)) != cudaSuccess) return err;
-        k_majority_rows<ASYNC, WK><<<blocks, kMajThreads, 0, st>>>(s, bin, flag);
+    if (mode == MODE_ASYNC && bin == 1) {
+        if ((err = wave_of(k_majority_lane<WK>, kMajThreads, sms, &blocks)) != cudaSuccess) return err;
+        k_majority_lane<WK><<<blocks, kMajThreads, 0, st>>>(s, 1);
+    } else if (mode == MODE_ASYNC && bin < kBins - 1) {
+        if ((err = wave_of(k_majority_rows<WK>, kMajThreads, sms, &blocks)) != cudaSuccess) return err;
+        k_majority_rows<WK><<<blocks, kMajThreads, 0, st>>>(s, bin, 1);
+    } else if (mode == MODE_ASYNC) {
+        if ((err = wave_of(k_majority_block<WK>, kMajThreads, sms, &blocks)) != cudaSuccess) return err;
+        k_majority_block<WK><<<blocks, kMajThreads, 0, st>>>(s, bin, 1);
     } else {
-        if ((err = wave_of(k_majority_block<ASYNC, WK>, kMajLongThreads, sms, &blocks)) != cudaSuccess) return err;
-        k_majority_block<ASYNC, WK><<<blocks, kMajLongThreads, 0, st>>>(s, bin, flag);
+        if ((err = wave_of(k_majority_all<WK>, kMajThreads, sms, &blocks)) != cudaSuccess) return err;
+        k_majority_all<WK><<<blocks, kMajThreads, 0, st>>>(s, mode != MODE_SYNC_FULL);
     }
     return cudaGetLastError();
 }
 
-template <bool ASYNC>
-static cudaError_t launch_majority_w(const DevState& s, int bin, int flag, cudaStream_t st, int sms) {
-    switch (s.weight_kind) {
-        case W_UNIT: return launch_majority_t<ASYNC, W_UNIT>(s, bin, flag, st, sms);
-        case W_U32: return launch_majority_t<ASYNC, W_U32>(s, bin, flag, st, sms);
-        case W_U8: return launch_majority_t<ASYNC, W_U8>(s, bin, flag, st, sms);
-        default: return launch_majority_t<ASYNC, W_F32>(s, bin, flag, st, sms);
-    }
-}
-
 cudaError_t launch_majority(const DevState& s, int mode, int bin, cudaStream_t st, int sms) {
     const int base = mode & ~kModeNonstrict;
-    const int flag = base != MODE_SYNC_FULL;
-    return base == MODE_ASYNC ? launch_majority_w<true>(s, bin, flag, st, sms)
-                              : launch_majority_w<false>(s, bin, flag, st, sms);
+    switch (s.weight_kind) {
+        case W_UNIT: return launch_majority_w<W_UNIT>(s, base, bin, st, sms);
+        case W_U32: return launch_majority_w<W_U32>(s, base, bin, st, sms);
+        case W_U8: return launch_majority_w<W_U8>(s, base, bin, st, sms);
+        default: return launch_majority_w<W_F32>(s, base, bin, st, sms);
+    }
 }
 
 }  // namespace lpa
