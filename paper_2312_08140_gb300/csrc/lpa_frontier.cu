@@ -504,6 +504,7 @@ __device__ void control_step(const DevState& s, int mode, int role, int dense_ne
             int per_pass = 1;
             for (int q = 0; q < kBins; ++q) per_pass += s.bin_static[q] ? 1 : 0;
             if (s.bin_static[kBins - 1] && s.ovf_possible) per_pass += 4;   // plan, slices, partitions, rescan
+            if (mode != MODE_ASYNC && s.bin_static[1]) per_pass += s.long_rows == 2 ? 1 : 0;
             int majority = 0;               // once per sweep: sample, bits, rows (asynchronous: per bin)
             if (s.dom_bits) {
                 majority = 3;

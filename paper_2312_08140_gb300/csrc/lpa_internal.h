@@ -191,6 +191,7 @@ struct DevState {
     int32_t warp_max;
     int32_t mid_max;
     int32_t large_max;
+    int32_t long_rows;         // bin 1 may hold rows too long for a lane: 1 scanned by k_sweep_lane, 2 by k_sweep_long
     int32_t warp_slots;        // per-warp table slots = next pow2 >= 2 * warp_max
     int32_t block_slots[kBlockBins];   // per-block shared table slots of bins 2..4
     float weight_max;          // largest weight (1 for unit weights)
@@ -238,9 +239,18 @@ cudaError_t launch_set_params(Ctrl* ctrl, double tau, int max_iters, int mode, i
                               int32_t* labels_out, int local_ids, cudaStream_t st);
 cudaError_t launch_sweep_small(const DevState& s, int mode, cudaStream_t st, int sms);
 // Bin 1: a warp per vertex in the asynchronous mode, a lane per vertex in the
-// synchronous ones.
+// synchronous ones (rows of at most kLaneEntries entries always fit a lane).
+constexpr int kLaneEntries = 61;
 cudaError_t launch_sweep_warp(const DevState& s, int mode, cudaStream_t st, int sms);
-cudaError_t launch_sweep_lane(const DevState& s, int mode, cudaStream_t st, int sms);
+// `fork` (may be null): during a capture, a second stream for the longer rows.
+struct LaneFork {
+    cudaStream_t st = nullptr;
+    cudaEvent_t begin = nullptr, end = nullptr;
+};
+cudaError_t launch_sweep_lane(const DevState& s, int mode, cudaStream_t st, int sms, const LaneFork* fork);
+// DevState::long_rows for weights, N and warp_max as in s and rows of at most
+// max_degree entries.
+int lane_long_rows(const DevState& s, int64_t max_degree);
 // Majority kernels (lpa_sweep_majority.cu), for single graphs whose block bins
 // hold kMajorityEntries: launch_dominant looks for a label that dominates the
 // pass and marks its vertices; launch_majority then settles the rows that it

@@ -311,6 +311,7 @@ cudaError_t run_cycle(lpa_server* S, int64_t entries, int64_t max_degree, bool f
     const int64_t limit[kBins] = {0, s.small_max, s.warp_max, s.mid_max, s.large_max};
     // only longer rows can overflow the last bin's table
     s.ovf_possible = 2 * max_degree > kLargeSlots ? 1 : 0;
+    s.long_rows = lane_long_rows(s, max_degree);
     cudaError_t e = cudaSuccess;
     for (int p = 0; p < passes && e == cudaSuccess; ++p) {
         // compaction: the cycle's frontier, then (async) the catch-up set
@@ -318,7 +319,7 @@ cudaError_t run_cycle(lpa_server* S, int64_t entries, int64_t max_degree, bool f
         if (e == cudaSuccess) e = launch_sweep_small(s, sweep_mode, st, S->sms);
         if (e == cudaSuccess && max_degree > limit[1])
             e = mode == MODE_ASYNC ? launch_sweep_warp(s, mode, st, S->sms)
-                                   : launch_sweep_lane(s, sweep_mode, st, S->sms);
+                                   : launch_sweep_lane(s, sweep_mode, st, S->sms, nullptr);
         for (int b = 2; b < kBins && e == cudaSuccess; ++b)
             if (max_degree > limit[b]) e = launch_sweep_block(s, sweep_mode, b, S->sms, st);
     }

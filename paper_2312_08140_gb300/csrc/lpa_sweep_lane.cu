@@ -26,15 +26,17 @@
 // 0.81, a lane per row with a hash table of its own 0.96 (8 warps per SM), with
 // all pairs compared 0.75, this kernel 0.39 (141 G entries/s; the gathers alone
 // take 0.18 at the 296 G/s of L2).  It is bound by instructions and their
-// latency at 20 warps per SM; 24 warps at 85 registers spill (0.46).
+// latency at 16 to 20 warps per SM; 24 warps at 85 registers spill (0.46).
 //
 // Keys (chosen at the launch from the number of vertices and the largest
 // weight): the label alone for unit weights; label and weight where both fit
 // 32 bits; else label and place in the row (6 bits), the weights waiting in
 // shared memory -- also for fp32 weights, whose sums are so taken in the row's
-// entry order.  Graphs whose labels leave no room for that, rows of more than
-// 64 entries and the few rows at the very end of the index array (a 16-byte
-// load would pass it) are taken by a whole warp each (lpa_warp_row.cuh).
+// entry order.  Longer rows (more than 64 slots) and the few rows at the very end
+// of the index array (a 16-byte load would pass it) are taken by a whole warp
+// each (lpa_warp_row.cuh): within k_sweep_lane where the key is the label or
+// holds the weight, else by a kernel of their own, k_sweep_long (see there), which
+// also takes every row of graphs whose labels leave no room for a key.
 //
 // The 32 rows of a step cost as much as the longest of them, so each warp
 // sorts the vertices of its part of the frontier into queues by row length and
@@ -53,6 +55,7 @@ namespace lpa {
 constexpr int kSortSlots = 32;          // row slots sorted at a time
 constexpr int kLaneMax = 64;            // row slots a lane can take
 constexpr int kPosBits = 6;             // log2(kLaneMax)
+static_assert(kLaneEntries + 3 == kLaneMax, "a row may start up to 3 slots past a 16-byte boundary");
 constexpr int kLaneQueues = 3;          // rows of up to 32 slots, of up to 64, longer ones
 constexpr int kLong = kLaneQueues - 1;
 constexpr int kLaneQueueCap = 64;       // a queue is drained before it can pass 31 + 32
@@ -63,7 +66,6 @@ enum LaneKey : int {
     KEY_LABEL = 0,      // label (unit weights)
     KEY_PACKED = 1,     // label << weight_bits | weight
     KEY_PLACE = 2,      // label << kPosBits | place in the row
-    KEY_NONE = 3,       // neither fits: every row by a whole warp
 };
 
 // ---- Batcher's odd-even merge sorting network for N keys -------------------
@@ -132,7 +134,7 @@ struct LaneRow {
     int32_t v, d;
     int64_t st;
 };
-__device__ __forceinline__ uint4 pack_row(const LaneRow& r) {      // st < 2^48, d < 2^16 (long rows re-read theirs)
+__device__ __forceinline__ uint4 pack_row(const LaneRow& r) {      // st < 2^48, d <= warp_max <= 256
     return make_uint4(r.k, (uint32_t)r.v, (uint32_t)r.st, (uint32_t)((uint64_t)r.st >> 32) | ((uint32_t)r.d << 16));
 }
 __device__ __forceinline__ LaneRow unpack_row(const uint4& q) {
@@ -301,8 +303,122 @@ __device__ __forceinline__ int32_t lane_pick(const DevState& s, const int32_t* C
     return (int32_t)best_lab;
 }
 
+// First sweep of a repeat-free graph: every label is still its vertex's id and
+// occurs once in a row, so the pick is the row's heaviest entry.  A lane per row,
+// straight from the list.  All threads of the block must call, once, as the last
+// step of the kernel.
+template <int WK, bool NS>
+__device__ __forceinline__ void identity_rows(const DevState& s, const Labels& L, const BinView& bv, bool marks,
+                                              uint32_t sweep, int64_t E_al) {
+    using T = typename Acc<WK>::T;
+    const unsigned cnt = bv.cnt;
+    unsigned long long my_changed = 0, my_changed_entries = 0;
+    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < cnt; k += gridDim.x * blockDim.x) {
+        const int32_t v = bv.list[k];
+        const int64_t st = s.off[v], en = s.off_end[v];
+        const int32_t own = L.C[v];
+        int32_t best = -1;
+        if (WK == W_UNIT && !NS) {
+            // equal weights and ascending neighbours: the first entry that
+            // is not v itself
+            for (int64_t e = st; e < en && best < 0; ++e) {
+                const int32_t j = __ldg(s.idx + e);
+                if (j != v) best = initial_label(s, j);
+            }
+        } else {
+            const TieRule tr = tie_rule(s, NS, sweep, v);
+            uint32_t key = 0, tie = 0xffffffffu;
+            for (int64_t a = st & ~(int64_t)3; a < en; a += 4) {
+                int32_t j[4];
+                T w[4];
+                load_row4<WK>(s, a, st, en, E_al, v, j, w);
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    if (j[c] != v) offer_candidate<T>(tr, w[c], initial_label(s, j[c]), key, tie);
+            }
+            if (key != 0u) best = tr.label(tie);
+        }
+        const bool changed = best >= 0 && best != own;
+        record_label<false>(L, bv.chg + k, v, own, best, changed);
+        if (changed) {
+            ++my_changed;
+            my_changed_entries += (unsigned)(en - st);
+            if (marks)
+                for (int64_t e = st; e < en; ++e) {
+                    const int32_t j = __ldg(s.idx + e);
+                    if (j != v) mark_unprocessed(s.flags, j);
+                }
+        }
+    }
+    flush_bin_counts(s, 1, my_changed, my_changed_entries);
+}
+
+// A row that a lane cannot take.
+__device__ __forceinline__ bool is_long(int64_t st, int64_t en, int64_t E_al) {
+    return en - (st & ~(int64_t)3) > kLaneMax || en > E_al;
+}
+
+// Row of frontier entry `at`; true if it is a longer one (or `all`) of a graph
+// that still runs.
+__device__ __forceinline__ bool load_long(const DevState& s, const Labels& L, const BinView& bv, bool batch, unsigned at,
+                                          int64_t E_al, LaneRow& r, bool all = false) {
+    r.k = bv.slot(at);
+    r.v = bv.list[r.k];
+    r.st = s.off[r.v];
+    const int64_t en = s.off_end[r.v];
+    r.d = (int)(en - r.st);
+    if (!all && !is_long(r.st, en, E_al)) return false;
+    if (batch && s.done[s.gid[r.v]]) {
+        const int32_t own = L.C[r.v];               // a done graph's vertex keeps its label
+        record_label<false>(L, bv.chg + r.k, r.v, own, own, false);
+        return false;
+    }
+    return true;
+}
+
+// After a warp scanned vertex v of row [st, en) (frontier slot k): its label, the
+// counts, and its neighbours' marks.  All 32 lanes must call.
+__device__ __forceinline__ void finish_long(const DevState& s, const Labels& L, const BinView& bv, bool batch, bool marks,
+                                            unsigned k, int32_t v, int64_t st, int64_t en, int32_t own, int32_t best,
+                                            unsigned long long& my_changed, unsigned long long& my_changed_entries) {
+    const unsigned lane = lane_id();
+    const bool changed = best >= 0 && best != own;      // warp-uniform
+    if (lane == 0) {
+        record_label<false>(L, bv.chg + k, v, own, best, changed);
+        if (changed) {
+            ++my_changed;
+            my_changed_entries += (unsigned long long)(en - st);
+            if (batch) atomicAdd(&s.dN[s.gid[v]], 1ull);
+        }
+    }
+    if (changed && marks) {
+        for (int64_t e0 = st + lane; e0 < en; e0 += 128) {
+            int32_t jj[4];
+            uint8_t f[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) jj[u] = e0 + 32 * u < en ? s.idx[e0 + 32 * u] : v;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) f[u] = jj[u] != v ? __ldcg(s.flags + jj[u]) : (uint8_t)1;
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (f[u] == 0) s.flags[jj[u]] = 1;
+        }
+    }
+}
+
+// Blocks per SM that the registers are to allow.  Rows are sorted faster by 16
+// warps with 128 registers each than by 20 with 96 (one sort after another: planted
+// partitions of 130,000 vertices, unit weights 389 -> 352 us a run, weights 1..4
+// 578 -> 542; 256 of them in a batch 20.18 -> 19.87 ms), except where the weight
+// columns leave room for 12 warps only (fp32, 1 M vertices: 8.94 ms at up to 168
+// registers, 8.82 at 128, 8.69 at 96).
+template <int KM>
+constexpr int kLaneBlocks = KM == KEY_PLACE ? 5 : 4;
+
+// take_long: rows that no lane can take are 0: left to k_sweep_long, 1: few,
+// scanned by the warp that meets them, 2: shared out where warps are to spare.
 template <int KM, int WK, bool NS>
-__global__ void __launch_bounds__(kLaneWarps * 32) k_sweep_lane(DevState s, int flag_neighbours) {
+__global__ void __launch_bounds__(kLaneWarps * 32, kLaneBlocks<KM>) k_sweep_lane(DevState s, int flag_neighbours, int take_long) {
     using T = typename Acc<WK>::T;
     using Sh = LaneShape<KM, WK>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -318,7 +434,6 @@ __global__ void __launch_bounds__(kLaneWarps * 32) k_sweep_lane(DevState s, int 
     const Labels L = labels_of(s);
     const bool marks = marks_on(s, flag_neighbours);
     const uint32_t sweep = NS ? (uint32_t)s.ctrl->iter + 1u : 0u;   // non-strict tie-break (Section 4.1.5)
-    const bool ident = !batch && identity_sweep<false, false>(s);
     const unsigned cnt = bv.cnt;
     const int64_t E_al = s.E & ~(int64_t)3;                                // 16-byte loads end here
     unsigned long long my_changed = 0, my_changed_entries = 0;
@@ -332,7 +447,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32) k_sweep_lane(DevState s, int 
         const int32_t own = act ? L.C[v] : 0;
         const TieRule tr = tie_rule(s, NS && act, sweep, v);
         int32_t best = -1;
-        if constexpr (KM != KEY_NONE) best = lane_pick<KM, WK, NS>(s, L.C, v, st, d, tr, halves, col, wts);
+        best = lane_pick<KM, WK, NS>(s, L.C, v, st, d, tr, halves, col, wts);
         const bool changed = act && best >= 0 && best != own;
         if (act) record_label<false>(L, bv.chg + k, v, own, best, changed);
         if (changed) {
@@ -361,89 +476,26 @@ __global__ void __launch_bounds__(kLaneWarps * 32) k_sweep_lane(DevState s, int 
 
     // The whole warp scans the vertex of one queue entry.
     auto long_step = [&](const LaneRow& r) {
-        const unsigned k = r.k;
         const int32_t v = r.v;
-        const int64_t st = r.st, en = s.off_end[v];
+        const int64_t st = r.st, en = st + r.d;
         const int32_t own = L.C[v];
-        const int d = (int)(en - st);
         const TieRule tr = tie_rule(s, NS, sweep, v);
         uint32_t key = 0, tie = 0xffffffffu;
-        const int32_t j = (int)lane < d ? load_index_keep(s.idx, st + lane) : v;
+        const int32_t j = (int)lane < r.d ? load_index_keep(s.idx, st + lane) : v;
         const bool ok = j != v;
-        const int32_t lab = ok ? load_label<false>(L.C, j) : kEmptyKey;
-        const T w = ok ? load_weight<WK>(s.w, st + lane) : (T)0;
+        const int32_t lab[1] = {ok ? load_label<false>(L.C, j) : kEmptyKey};
+        const T w[1] = {ok ? load_weight<WK>(s.w, st + lane) : (T)0};
         int32_t* keys = reinterpret_cast<int32_t*>(mem);
         T* vals = reinterpret_cast<T*>(keys + 512);
         warp_long_row<false, WK>(s, L, keys, vals, reinterpret_cast<unsigned*>(vals + 512), 9, tr, st, en, v, lab, w, key,
                                  tie);
         const uint32_t best_key = warp_argmax_tie(key, tie);
         const int32_t best = best_key == 0xffffffffu ? -1 : tr.label(best_key);
-        const bool changed = best >= 0 && best != own;      // warp-uniform
-        if (lane == 0) {
-            record_label<false>(L, bv.chg + k, v, own, best, changed);
-            if (changed) {
-                ++my_changed;
-                my_changed_entries += (unsigned)d;
-                if (batch) atomicAdd(&s.dN[s.gid[v]], 1ull);
-            }
-        }
-        if (changed && marks) {
-            for (int64_t e0 = st + lane; e0 < en; e0 += 128) {
-                int32_t jj[4];
-                uint8_t f[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) jj[u] = e0 + 32 * u < en ? s.idx[e0 + 32 * u] : v;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) f[u] = jj[u] != v ? __ldcg(s.flags + jj[u]) : (uint8_t)1;
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (f[u] == 0) s.flags[jj[u]] = 1;
-            }
-        }
+        finish_long(s, L, bv, batch, marks, r.k, v, st, en, own, best, my_changed, my_changed_entries);
     };
 
-    // First sweep of a repeat-free graph: every label is still its vertex's id
-    // and occurs once in a row, so the pick is the row's heaviest entry.  A
-    // lane per row, straight from the list.
-    if (ident) {
-        for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < cnt; k += gridDim.x * blockDim.x) {
-            const int32_t v = bv.list[k];
-            const int64_t st = s.off[v], en = s.off_end[v];
-            const int32_t own = L.C[v];
-            int32_t best = -1;
-            if (WK == W_UNIT && !NS) {
-                // equal weights and ascending neighbours: the first entry that
-                // is not v itself
-                for (int64_t e = st; e < en && best < 0; ++e) {
-                    const int32_t j = __ldg(s.idx + e);
-                    if (j != v) best = initial_label(s, j);
-                }
-            } else {
-                const TieRule tr = tie_rule(s, NS, sweep, v);
-                uint32_t key = 0, tie = 0xffffffffu;
-                for (int64_t a = st & ~(int64_t)3; a < en; a += 4) {
-                    int32_t j[4];
-                    T w[4];
-                    load_row4<WK>(s, a, st, en, E_al, v, j, w);
-#pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                        if (j[c] != v) offer_candidate<T>(tr, w[c], initial_label(s, j[c]), key, tie);
-                }
-                if (key != 0u) best = tr.label(tie);
-            }
-            const bool changed = best >= 0 && best != own;
-            record_label<false>(L, bv.chg + k, v, own, best, changed);
-            if (changed) {
-                ++my_changed;
-                my_changed_entries += (unsigned)(en - st);
-                if (marks)
-                    for (int64_t e = st; e < en; ++e) {
-                        const int32_t j = __ldg(s.idx + e);
-                        if (j != v) mark_unprocessed(s.flags, j);
-                    }
-            }
-        }
-        flush_bin_counts(s, 1, my_changed, my_changed_entries);
+    if (!batch && identity_sweep<false, false>(s)) {
+        identity_rows<WK, NS>(s, L, bv, marks, sweep, E_al);
         return;
     }
 
@@ -453,6 +505,25 @@ __global__ void __launch_bounds__(kLaneWarps * 32) k_sweep_lane(DevState s, int 
     const unsigned nchunks = (cnt + 31u) / 32u;
     const unsigned nwarps = gridDim.x * kLaneWarps;
     unsigned chunk = (unsigned)wib * gridDim.x + blockIdx.x;
+    unsigned n[kLaneQueues];
+#pragma unroll
+    for (int q = 0; q < kLaneQueues; ++q) n[q] = 0u;
+    // Where at least half of the warps have no chunk, these read the frontier a
+    // second time and take its longer rows, one part of at most 32 entries each
+    // (otherwise the rows of a chunk are scanned one after another: 2,000 vertices
+    // of degree 90, unit weights, 5 sweeps: 320 us, so 110).
+    const bool shared_out = take_long == 2 && nchunks * 2u <= nwarps;
+    if (shared_out && chunk >= nchunks) {
+        const unsigned others = nwarps - nchunks, width = (cnt + others - 1u) / others;     // <= 32
+        const unsigned k = (chunk - nchunks) * width + lane;
+        LaneRow r{};
+        const bool mine = lane < width && k < cnt && load_long(s, L, bv, batch, k, E_al, r);
+        const unsigned m = __ballot_sync(kFull, mine);
+        if (mine) queue[kLong * kLaneQueueCap + __popc(m & lanes_below())] = pack_row(r);
+        n[kLong] = __popc(m);
+        __syncwarp();
+    }
+    const bool longs = take_long && !shared_out;
     unsigned k_c = 0, k_n = 0;                      // their slots in the frontier list
     auto vertex_of = [&](unsigned c, unsigned& slot) -> int32_t {
         const unsigned k = c * 32u + lane;
@@ -471,9 +542,6 @@ __global__ void __launch_bounds__(kLaneWarps * 32) k_sweep_lane(DevState s, int 
         }
     };
     load_row();
-    unsigned n[kLaneQueues];
-#pragma unroll
-    for (int q = 0; q < kLaneQueues; ++q) n[q] = 0u;
     for (;;) {
         bool full = false;
 #pragma unroll
@@ -487,9 +555,9 @@ __global__ void __launch_bounds__(kLaneWarps * 32) k_sweep_lane(DevState s, int 
             r.d = (int)(en_c - st_c);
             int cls = -1;
             if (v_c >= 0) {
-                const int span = (int)(en_c - (st_c & ~(int64_t)3));
-                cls = KM == KEY_NONE || span > kLaneMax || en_c > E_al ? kLong : span <= kSortSlots ? 0 : 1;
-                if (batch && done_c) {
+                cls = is_long(st_c, en_c, E_al) ? kLong : en_c - (st_c & ~(int64_t)3) <= kSortSlots ? 0 : 1;
+                if (cls == kLong && !longs) cls = -1;               // other warps take it
+                if (batch && done_c && cls >= 0) {
                     cls = -1;                       // a done graph's vertex keeps its label
                     const int32_t own = L.C[v_c];
                     record_label<false>(L, bv.chg + r.k, v_c, own, own, false);
@@ -540,9 +608,141 @@ __global__ void __launch_bounds__(kLaneWarps * 32) k_sweep_lane(DevState s, int 
     flush_bin_counts(s, 1, my_changed, my_changed_entries);
 }
 
+// ---- longer rows, a warp per row -------------------------------------------
+// The rows that no lane can take, or (`all`) every row of the bin.  Each warp
+// goes through chunks of the frontier, as small as gives every warp one, and
+// collects their longer rows in a queue; while one row is scanned, the labels and
+// weights of the next one's first kAhead x 32 entries and the ids of the one after
+// that are on their way (labels do not change during a synchronous sweep).
+//
+// fp32 rows spend their time in the table (a claim, a lane mask and ordered sums
+// per chunk of 32 entries), one row's steps waiting for each other, so it takes
+// warps to hide them: inside k_sweep_lane, whose weight columns leave room for 12
+// warps per SM, planted partitions of 200,000 vertices and mean degree 80 took
+// 4.23 ms a run, here 2.51 (a warp per row with table atomics for every row of the
+// bin, before k_sweep_lane came: 2.86).
+constexpr int kLongWarps = 8;           // per block
+constexpr int kAhead = 4;
+
+template <int WK, bool NS>
+__global__ void __launch_bounds__(kLongWarps * 32, 3) k_sweep_long(DevState s, int flag_neighbours, int all) {
+    using T = typename Acc<WK>::T;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const unsigned lane = lane_id();
+    const int wib = threadIdx.x >> 5;
+    const bool batch = s.G > 1;
+    const bool ident = !batch && identity_sweep<false, false>(s);
+    if (ident && !all) return;                      // k_sweep_lane took every row
+    const unsigned slots = (unsigned)s.warp_slots;
+    const int log_slots = ceil_log2(slots);
+    const size_t warp_bytes = kLaneQueueCap * sizeof(uint4) + (size_t)slots * 4 * kTableWords<WK>;
+    uint4* queue = reinterpret_cast<uint4*>(smem_raw + (size_t)wib * warp_bytes);
+    int32_t* keys = reinterpret_cast<int32_t*>(queue + kLaneQueueCap);
+    T* vals = reinterpret_cast<T*>(keys + slots);
+    unsigned* peers_of = reinterpret_cast<unsigned*>(vals + slots);
+    for (unsigned q = lane; q < slots * kTableWords<WK>; q += 32) keys[q] = q < slots ? kEmptyKey : 0;
+
+    const BinView bv = bin_view(s, 1);
+    const Labels L = labels_of(s);
+    const bool marks = marks_on(s, flag_neighbours);
+    const uint32_t sweep = NS ? (uint32_t)s.ctrl->iter + 1u : 0u;   // non-strict tie-break (Section 4.1.5)
+    const unsigned cnt = bv.cnt;
+    const int64_t E_al = s.E & ~(int64_t)3;
+    if (ident) {
+        identity_rows<WK, NS>(s, L, bv, marks, sweep, E_al);
+        return;
+    }
+    unsigned long long my_changed = 0, my_changed_entries = 0;
+
+    auto load_ids = [&](const LaneRow& r, int32_t (&j)[kAhead]) {
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u)
+            j[u] = 32 * u + (int)lane < r.d ? load_index_keep(s.idx, r.st + 32 * u + lane) : r.v;
+    };
+    auto load_labels = [&](const LaneRow& r, const int32_t (&j)[kAhead], int32_t& own, int32_t (&lab)[kAhead],
+                           T (&w)[kAhead]) {
+        own = L.C[r.v];
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            const bool ok = j[u] != r.v;
+            lab[u] = ok ? load_label<false>(L.C, j[u]) : kEmptyKey;
+            w[u] = ok ? load_weight<WK>(s.w, r.st + 32 * u + lane) : (T)0;
+        }
+    };
+    // the queue's `rows` vertices, one after another
+    auto scan_queue = [&](unsigned rows) {
+        LaneRow now = unpack_row(queue[0]), next = unpack_row(queue[rows > 1u ? 1 : 0]);
+        int32_t ids[kAhead], lab[kAhead], own = 0;
+        T w[kAhead];
+        load_ids(now, ids);
+        load_labels(now, ids, own, lab, w);
+        load_ids(next, ids);
+#pragma unroll 1
+        for (unsigned i = 0; i < rows; ++i) {
+            int32_t next_lab[kAhead], next_own = 0;
+            T next_w[kAhead];
+            load_labels(next, ids, next_own, next_lab, next_w);
+            const LaneRow after = unpack_row(queue[min(i + 2u, rows - 1u)]);
+            load_ids(after, ids);
+            const TieRule tr = tie_rule(s, NS, sweep, now.v);
+            uint32_t key = 0, tie = 0xffffffffu;
+            const int64_t en = now.st + now.d;
+            warp_long_row<false, WK>(s, L, keys, vals, peers_of, log_slots, tr, now.st, en, now.v, lab, w, key, tie);
+            const uint32_t best_key = warp_argmax_tie(key, tie);
+            const int32_t best = best_key == 0xffffffffu ? -1 : tr.label(best_key);
+            finish_long(s, L, bv, batch, marks, now.k, now.v, now.st, en, own, best, my_changed, my_changed_entries);
+            now = next;
+            next = after;
+            own = next_own;
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) {
+                lab[u] = next_lab[u];
+                w[u] = next_w[u];
+            }
+        }
+        __syncwarp();
+    };
+
+    const unsigned nwarps = gridDim.x * kLongWarps;
+    const unsigned width = max(1u, min(32u, (cnt + nwarps - 1u) / nwarps));
+    const unsigned nchunks = (cnt + width - 1u) / width;
+    unsigned n = 0;                                 // rows in the queue
+    for (unsigned chunk = (unsigned)wib * gridDim.x + blockIdx.x; chunk < nchunks; chunk += nwarps) {
+        const unsigned at = chunk * width + lane;
+        LaneRow r{};
+        const bool mine = lane < width && at < cnt && load_long(s, L, bv, batch, at, E_al, r, all != 0);
+        const unsigned m = __ballot_sync(kFull, mine);
+        if (mine) queue[n + __popc(m & lanes_below())] = pack_row(r);
+        n += __popc(m);
+        __syncwarp();
+        if (n >= 32u) {
+            scan_queue(n);
+            n = 0;
+        }
+    }
+    if (n > 0u) scan_queue(n);
+    flush_bin_counts(s, 1, my_changed, my_changed_entries);
+}
+
+template <int WK, bool NS>
+static cudaError_t launch_long_k(const DevState& s, int flag, int all, cudaStream_t st, int sms) {
+    constexpr int threads = kLongWarps * 32;
+    const size_t smem = kLongWarps * (kLaneQueueCap * sizeof(uint4) + (size_t)s.warp_slots * 4 * kTableWords<WK>);
+    auto kern = k_sweep_long<WK, NS>;
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (err != cudaSuccess) return err;
+    int per_sm = 0;
+    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+    if (err != cudaSuccess) return err;
+    if (per_sm < 1) per_sm = 1;
+    kern<<<sms * per_sm, threads, smem, st>>>(s, flag, all);
+    return cudaGetLastError();
+}
+
 template <int KM, int WK, bool NS>
-static cudaError_t launch_lane_k(const DevState& s, int flag, cudaStream_t st, int sms) {
+static cudaError_t launch_lane_k(const DevState& s, int flag, cudaStream_t st, int sms, const LaneFork* fork) {
     constexpr int threads = kLaneWarps * 32;
+    const bool apart = KM == KEY_PLACE && s.long_rows == 2;
     const size_t smem = kLaneWarps * LaneShape<KM, WK>::WARP_BYTES;
     auto kern = k_sweep_lane<KM, WK, NS>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -551,38 +751,68 @@ static cudaError_t launch_lane_k(const DevState& s, int flag, cudaStream_t st, i
     err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
     if (err != cudaSuccess) return err;
     if (per_sm < 1) per_sm = 1;
-    kern<<<sms * per_sm, threads, smem, st>>>(s, flag);
-    return cudaGetLastError();
+    // the two kernels write different vertices, so a graph runs them side by side
+    // (one after the other, a batch of 64 planted partitions, 3.2 M entries, fp32
+    // weights, lost 4 of 32 us a sweep)
+    const bool beside = apart && fork != nullptr;
+    if (beside) {
+        if ((err = cudaEventRecord(fork->begin, st)) != cudaSuccess) return err;
+        if ((err = cudaStreamWaitEvent(fork->st, fork->begin, 0)) != cudaSuccess) return err;
+    }
+    kern<<<sms * per_sm, threads, smem, st>>>(s, flag, apart ? 0 : s.long_rows ? 2 : 1);
+    err = cudaGetLastError();
+    if constexpr (KM == KEY_PLACE) {
+        if (err == cudaSuccess && apart) err = launch_long_k<WK, NS>(s, flag, 0, beside ? fork->st : st, sms);
+    }
+    if (beside) {
+        if (err == cudaSuccess) err = cudaEventRecord(fork->end, fork->st);
+        if (err == cudaSuccess) err = cudaStreamWaitEvent(st, fork->end, 0);
+    }
+    return err;
 }
 
 template <int KM, int WK>
-static cudaError_t launch_lane_t(const DevState& s, int flag, int ns, cudaStream_t st, int sms) {
-    return ns ? launch_lane_k<KM, WK, true>(s, flag, st, sms) : launch_lane_k<KM, WK, false>(s, flag, st, sms);
+static cudaError_t launch_lane_t(const DevState& s, int flag, int ns, cudaStream_t st, int sms, const LaneFork* fork) {
+    return ns ? launch_lane_k<KM, WK, true>(s, flag, st, sms, fork) : launch_lane_k<KM, WK, false>(s, flag, st, sms, fork);
+}
+
+// The key layout of the graph's rows, -1 if none fits.
+static int key_of(const DevState& s) {
+    if (s.weight_kind == W_UNIT) return KEY_LABEL;
+    if (s.weight_kind != W_F32 && s.weight_bits > 0 && s.weight_bits < 32 && s.N < (1ll << (32 - s.weight_bits)))
+        return KEY_PACKED;
+    // 16-byte loads of 4-byte weights (the caller's own array may start anywhere)
+    const bool aligned = s.weight_kind == W_U8 || (reinterpret_cast<uintptr_t>(s.w) & 15u) == 0;
+    return aligned && s.N < (1ll << (32 - kPosBits)) ? KEY_PLACE : -1;
+}
+
+int lane_long_rows(const DevState& s, int64_t max_degree) {
+    if (max_degree <= kLaneEntries || s.warp_max <= kLaneEntries) return 0;
+    return key_of(s) == KEY_PLACE ? 2 : 1;
 }
 
 template <int WK>
-static cudaError_t launch_lane_w(const DevState& s, int flag, int ns, cudaStream_t st, int sms) {
+static cudaError_t launch_lane_w(const DevState& s, int flag, int ns, cudaStream_t st, int sms, const LaneFork* fork) {
     if constexpr (WK == W_UNIT) {
-        return launch_lane_t<KEY_LABEL, WK>(s, flag, ns, st, sms);
+        return launch_lane_t<KEY_LABEL, WK>(s, flag, ns, st, sms, fork);
     } else {
-        // 16-byte loads of 4-byte weights (the caller's own array may start anywhere)
-        const bool aligned = WK == W_U8 || (reinterpret_cast<uintptr_t>(s.w) & 15u) == 0;
-        if constexpr (WK == W_U8 || WK == W_U32)
-            if (s.weight_bits > 0 && s.weight_bits < 32 && s.N < (1ll << (32 - s.weight_bits)))
-                return launch_lane_t<KEY_PACKED, WK>(s, flag, ns, st, sms);
-        if (aligned && s.N < (1ll << (32 - kPosBits))) return launch_lane_t<KEY_PLACE, WK>(s, flag, ns, st, sms);
-        return launch_lane_t<KEY_NONE, WK>(s, flag, ns, st, sms);
+        const int key = key_of(s);
+        if constexpr (WK != W_F32) {
+            if (key == KEY_PACKED) return launch_lane_t<KEY_PACKED, WK>(s, flag, ns, st, sms, fork);
+        }
+        if (key == KEY_PLACE) return launch_lane_t<KEY_PLACE, WK>(s, flag, ns, st, sms, fork);
+        return ns ? launch_long_k<WK, true>(s, flag, 1, st, sms) : launch_long_k<WK, false>(s, flag, 1, st, sms);
     }
 }
 
-cudaError_t launch_sweep_lane(const DevState& s, int mode, cudaStream_t st, int sms) {
+cudaError_t launch_sweep_lane(const DevState& s, int mode, cudaStream_t st, int sms, const LaneFork* fork) {
     const int ns = (mode & kModeNonstrict) != 0;
     const int flag = (mode & ~kModeNonstrict) != MODE_SYNC_FULL;
     switch (s.weight_kind) {
-        case W_UNIT: return launch_lane_w<W_UNIT>(s, flag, ns, st, sms);
-        case W_U32: return launch_lane_w<W_U32>(s, flag, ns, st, sms);
-        case W_U8: return launch_lane_w<W_U8>(s, flag, ns, st, sms);
-        default: return launch_lane_w<W_F32>(s, flag, ns, st, sms);
+        case W_UNIT: return launch_lane_w<W_UNIT>(s, flag, ns, st, sms, fork);
+        case W_U32: return launch_lane_w<W_U32>(s, flag, ns, st, sms, fork);
+        case W_U8: return launch_lane_w<W_U8>(s, flag, ns, st, sms, fork);
+        default: return launch_lane_w<W_F32>(s, flag, ns, st, sms, fork);
     }
 }
 

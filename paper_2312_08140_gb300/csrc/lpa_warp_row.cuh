@@ -106,10 +106,10 @@ __device__ __forceinline__ void offer_candidate(const TieRule& tr, T sum, int32_
     }
 }
 
-// Row [st, en) of vertex v (32 < en - st <= half the table's slots): this
-// lane's best (sum key, tie key).  lab0 and w0 are the labels and weights of
-// the first 32 entries (kEmptyKey: none).  The table is all free slots before
-// and after.  All 32 lanes must call.
+// Row [st, en) of vertex v (en - st at most half the table's slots, and 256):
+// this lane's best (sum key, tie key).  lab0[c] and w0[c] are the label and
+// weight of entry 32 c + lane (kEmptyKey: none), loaded by the caller.  The table
+// is all free slots before and after.  All 32 lanes must call.
 //
 // The label of the row's first entry is summed apart, by votes: once
 // communities form it is most often the label of nearly the whole row, and its
@@ -117,15 +117,16 @@ __device__ __forceinline__ void offer_candidate(const TieRule& tr, T sum, int32_
 // one word, against 2 for distinct words).  Entries of other labels go into
 // the table; each lane remembers the slots of its entries (16 bits per chunk
 // of 32 entries) and reads their sums when the row is complete.
-template <bool ASYNC, int WK>
+template <bool ASYNC, int WK, int K>
 __device__ __forceinline__ void warp_long_row(const DevState& s, const Labels& L, int32_t* keys,
                                               typename Acc<WK>::T* vals, [[maybe_unused]] unsigned* peers_of,
                                               int log_slots, const TieRule& tr, int64_t st, int64_t en, int32_t v,
-                                              int32_t lab0, typename Acc<WK>::T w0, uint32_t& key, uint32_t& tie) {
+                                              const int32_t (&lab0)[K], const typename Acc<WK>::T (&w0)[K],
+                                              uint32_t& key, uint32_t& tie) {
     using T = typename Acc<WK>::T;
     const unsigned lane = lane_id();
-    const unsigned okm = __ballot_sync(kFull, lab0 != kEmptyKey);
-    const int32_t lead = __shfl_sync(kFull, lab0, okm ? __ffs(okm) - 1 : 0);
+    const unsigned okm = __ballot_sync(kFull, lab0[0] != kEmptyKey);
+    const int32_t lead = __shfl_sync(kFull, lab0[0], okm ? __ffs(okm) - 1 : 0);
     T lead_sum = (T)0;
     uint64_t mine[2] = {~0ull, ~0ull};
     auto add_chunk = [&](int32_t lab, T w, int c) {
@@ -160,9 +161,11 @@ __device__ __forceinline__ void warp_long_row(const DevState& s, const Labels& L
             else mine[1] &= put;
         }
     };
-    add_chunk(lab0, w0, 0);
-    int c = 1;
-    for (int64_t e0 = st + 32; e0 < en; e0 += 32 * kWarpUnroll) {
+    int c = 0;
+#pragma unroll
+    for (int u = 0; u < K; ++u)
+        if (st + 32 * u < en) add_chunk(lab0[u], w0[u], c++);       // warp-uniform
+    for (int64_t e0 = st + 32 * K; e0 < en; e0 += 32 * kWarpUnroll) {
         int32_t jj[kWarpUnroll], ll[kWarpUnroll];
         T wq[kWarpUnroll];
 #pragma unroll
