@@ -25,14 +25,15 @@ def lpa():
     return m
 
 
-def weights(g, kind):
+def weights(g, kind, top=None):
     """Symmetric: a hash of the vertex pair; the largest weight occurs."""
+    top = top or TOP.get(kind)
     if kind == "unit":
         return None
     row = np.repeat(np.arange(g.n), np.diff(g.off))
     pair = (np.minimum(row, g.idx).astype(np.uint64) * np.uint64(g.n) + np.maximum(row, g.idx).astype(np.uint64))
-    w = 1 + ((pair * np.uint64(0x9E3779B97F4A7C15)) >> np.uint64(33)).astype(np.int64) % TOP[kind]
-    w[row + g.idx == row[0] + g.idx[0]] = TOP[kind]
+    w = 1 + ((pair * np.uint64(0x9E3779B97F4A7C15)) >> np.uint64(33)).astype(np.int64) % top
+    w[row + g.idx == row[0] + g.idx[0]] = top
     return w.astype(np.float32) / (4 if kind == "quarter" else 1)
 
 
