@@ -195,7 +195,10 @@ typedef struct {
 } lpa_config;
 
 /* Time per phase of one run, from CUDA events recorded around every launch
- * (lpa_run_profiled).  Times in milliseconds. */
+ * (lpa_run_profiled).  Times in milliseconds.  What precedes a sweep's bins -- on
+ * graphs with 4 M entries in the block bins the search for a dominating label
+ * and, in the synchronous modes, the rows of all bins that it settles -- counts
+ * to the bin launched first: the thread bin, asynchronously the last one. */
 typedef struct {
     int32_t iterations;
     int32_t reserved;
@@ -247,9 +250,11 @@ lpa_status lpa_tolerance_threshold(double tolerance, int64_t n, int64_t *out);
  * Validates the CSR on the device (returns LPA_ERR_INVALID_GRAPH on failure)
  * and synchronises `stream` before returning.  Device memory: the CSR copy
  * (unless borrowed) plus about 21 bytes per vertex of working state (two
- * label buffers, flags, the frontier bitmap, bin lists and change marks) and
- * 8 more per vertex once lpa_modularity has been called, taken from the
- * library's per-device memory pool; lpa_graph_props reports the total. */
+ * label buffers, flags, the frontier bitmap, bin lists and change marks), 4.1
+ * more per vertex on graphs with 4 M entries in the block bins (rows left by the
+ * majority kernels, which are done without if that much is not to be had) and 8
+ * more once lpa_modularity has been called, taken from the library's per-device
+ * memory pool; lpa_graph_props reports the total. */
 lpa_status lpa_graph_create(int64_t n, int64_t nnz, const int64_t *offsets, const int32_t *indices,
                             const float *weights, uint32_t flags, void *stream, lpa_graph_t *out);
 
