@@ -540,7 +540,9 @@ __device__ void control_step(const DevState& s, int mode, int role, int dense_ne
             if (mode != MODE_ASYNC && s.dense_permille <= 1000) {
                 const int from = s.active_entries <= kDenseEntries ? min(kDensePermille, s.dense_permille)
                                                                    : s.dense_permille;
-                skip = skip || changed * 1000.0 >= (double)from * active;
+                // (in integers: nothing runs beside this step, and an fp64 product
+                // takes it 0.1 us)
+                skip = skip || pass_changed * 1000ull >= (unsigned long long)from * (unsigned long long)s.active_entries;
             }
             c->skip_marks = skip && allow_dense ? 1 : 0;
             c->last_pass_high = high ? 1 : 0;
