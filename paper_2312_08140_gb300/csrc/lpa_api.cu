@@ -144,7 +144,6 @@ struct Engine {
     cudaGraph_t graph[6] = {};         // per mode, strict (0..2) and non-strict (3..5)
     cudaGraphExec_t exec[6] = {};
     cudaStream_t cap_top = nullptr, cap_body = nullptr;
-    LaneFork fork;                                 // second branch of a sweep's graph (build_graph)
     // modularity scratch
     double* Sigma = nullptr;
     ModAccum* acc = nullptr;
@@ -188,9 +187,6 @@ void engine_free(Engine& E) {
     destroy_graphs(E);
     if (E.cap_top) cudaStreamDestroy(E.cap_top);
     if (E.cap_body) cudaStreamDestroy(E.cap_body);
-    if (E.fork.st) cudaStreamDestroy(E.fork.st);
-    if (E.fork.begin) cudaEventDestroy(E.fork.begin);
-    if (E.fork.end) cudaEventDestroy(E.fork.end);
     if (E.ovf) E.owned.push_back(E.ovf);
     E.ovf = nullptr;
     for (void* p : E.ovf_scratch) E.owned.push_back(p);
@@ -586,8 +582,8 @@ cudaError_t launch_pass_start(Engine& E, int mode, cudaStream_t st) {
     return err;
 }
 
-// `main`: the sweep's main pass; `fork`: see launch_sweep_lane.
-cudaError_t launch_bin(Engine& E, int mode, int bin, bool main, const LaneFork* fork, cudaStream_t st) {
+// `main`: the sweep's main pass.
+cudaError_t launch_bin(Engine& E, int mode, int bin, bool main, cudaStream_t st) {
     if (main && E.s.dom_bits && bin >= 1 && (mode & ~kModeNonstrict) == MODE_ASYNC) {
         cudaError_t err = cudaSuccess;
         if (bin == 2 || bin == 3) err = launch_dominant(E.s, bin, st, E.sms);
@@ -597,7 +593,7 @@ cudaError_t launch_bin(Engine& E, int mode, int bin, bool main, const LaneFork* 
     if (bin == 0) return launch_sweep_small(E.s, mode, st, E.sms);
     if (bin == 1)
         return (mode & ~kModeNonstrict) == MODE_ASYNC ? launch_sweep_warp(E.s, mode, st, E.sms)
-                                                      : launch_sweep_lane(E.s, mode, st, E.sms, fork);
+                                                      : launch_sweep_lane(E.s, mode, st, E.sms);
     return launch_sweep_block(E.s, mode, bin, E.sms, st);
 }
 
@@ -622,7 +618,7 @@ cudaError_t enqueue_pass(Engine& E, int mode, bool main, cudaStream_t st) {
     for (int k = 0; k < kBins; ++k) {
         const int b = bin_at(mode, k);
         if (E.s.bin_static[b] == 0) continue;
-        cudaError_t err = launch_bin(E, mode, b, main, E.fork.st ? &E.fork : nullptr, st);
+        cudaError_t err = launch_bin(E, mode, b, main, st);
         if (err != cudaSuccess) return err;
     }
     return cudaSuccess;
@@ -698,14 +694,6 @@ lpa_status build_graph(Engine& E, int mode) {
     err = cudaStreamUpdateCaptureDependencies(E.cap_top, &cond, nullptr, 1, cudaStreamSetCaptureDependencies);
     if (err != cudaSuccess) return bail(err, "update capture deps");
     cudaGraph_t body = cp.conditional.phGraph_out[0];
-    if (E.s.long_rows == 2 && !E.fork.st) {
-        LaneFork f;
-        err = cudaEventCreateWithFlags(&f.begin, cudaEventDisableTiming);
-        if (err == cudaSuccess) err = cudaEventCreateWithFlags(&f.end, cudaEventDisableTiming);
-        if (err == cudaSuccess) err = cudaStreamCreateWithFlags(&f.st, cudaStreamNonBlocking);
-        E.fork = f;
-        if (err != cudaSuccess) return bail(err, "second capture stream");
-    }
     err = cudaStreamBeginCaptureToGraph(E.cap_body, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
     if (err != cudaSuccess) return bail(err, "begin capture (body)");
     if ((err = enqueue_sweep(E, mode, h, 1, E.cap_body)) != cudaSuccess) return bail(err, "sweep");
@@ -847,7 +835,7 @@ lpa_status engine_run_profiled(Engine& E, int mode, double tol, int32_t max_iter
                 LPA_P(cudaEventRecord(ev[k], st));
                 // (its time is the first bin's, so that the parts add up to the sweep)
                 if (p == 0 && k == 0) LPA_P(launch_pass_start(E, mode | (ns ? kModeNonstrict : 0), st));
-                if (E.s.bin_static[b]) LPA_P(launch_bin(E, mode | (ns ? kModeNonstrict : 0), b, p == 0, nullptr, st));
+                if (E.s.bin_static[b]) LPA_P(launch_bin(E, mode | (ns ? kModeNonstrict : 0), b, p == 0, st));
             }
             LPA_P(cudaEventRecord(ev[kBins], st));
             LPA_P(launch_finish(E.s, mode, p + 1 < passes ? kRoleCatchUp : kRoleEndSweep, none, 0, st, E.sms));

@@ -242,12 +242,7 @@ cudaError_t launch_sweep_small(const DevState& s, int mode, cudaStream_t st, int
 // synchronous ones (rows of at most kLaneEntries entries always fit a lane).
 constexpr int kLaneEntries = 61;
 cudaError_t launch_sweep_warp(const DevState& s, int mode, cudaStream_t st, int sms);
-// `fork` (may be null): during a capture, a second stream for the longer rows.
-struct LaneFork {
-    cudaStream_t st = nullptr;
-    cudaEvent_t begin = nullptr, end = nullptr;
-};
-cudaError_t launch_sweep_lane(const DevState& s, int mode, cudaStream_t st, int sms, const LaneFork* fork);
+cudaError_t launch_sweep_lane(const DevState& s, int mode, cudaStream_t st, int sms);
 // DevState::long_rows for weights, N and warp_max as in s and rows of at most
 // max_degree entries.
 int lane_long_rows(const DevState& s, int64_t max_degree);

@@ -319,7 +319,7 @@ cudaError_t run_cycle(lpa_server* S, int64_t entries, int64_t max_degree, bool f
         if (e == cudaSuccess) e = launch_sweep_small(s, sweep_mode, st, S->sms);
         if (e == cudaSuccess && max_degree > limit[1])
             e = mode == MODE_ASYNC ? launch_sweep_warp(s, mode, st, S->sms)
-                                   : launch_sweep_lane(s, sweep_mode, st, S->sms, nullptr);
+                                   : launch_sweep_lane(s, sweep_mode, st, S->sms);
         for (int b = 2; b < kBins && e == cudaSuccess; ++b)
             if (max_degree > limit[b]) e = launch_sweep_block(s, sweep_mode, b, S->sms, st);
     }

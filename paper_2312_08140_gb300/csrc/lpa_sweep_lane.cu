@@ -47,6 +47,7 @@
 // (Section 4.1.5).  A lane whose vertex changes walks the row again to mark
 // the neighbours unprocessed (Section 4.1.4).
 #include <utility>
+#include <vector>
 
 #include "lpa_warp_row.cuh"
 
@@ -411,14 +412,16 @@ __device__ __forceinline__ void finish_long(const DevState& s, const Labels& L, 
 // partitions of 130,000 vertices, unit weights 389 -> 352 us a run, weights 1..4
 // 578 -> 542; 256 of them in a batch 20.18 -> 19.87 ms), except where the weight
 // columns leave room for 12 warps only (fp32, 1 M vertices: 8.94 ms at up to 168
-// registers, 8.82 at 128, 8.69 at 96).
-template <int KM>
-constexpr int kLaneBlocks = KM == KEY_PLACE ? 5 : 4;
+// registers, 8.82 at 128, 8.69 at 96) and where longer rows, a warp each, want 20
+// (200,000 vertices of mean degree 120, unit weights: 1.96 ms with 16, 1.72).
+template <int KM, bool SHARE>
+constexpr int kLaneBlocks = KM == KEY_PLACE || SHARE ? 5 : 4;
 
-// take_long: rows that no lane can take are 0: left to k_sweep_long, 1: few,
-// scanned by the warp that meets them, 2: shared out where warps are to spare.
-template <int KM, int WK, bool NS>
-__global__ void __launch_bounds__(kLaneWarps * 32, kLaneBlocks<KM>) k_sweep_lane(DevState s, int flag_neighbours, int take_long) {
+// Rows that no lane can take are left to k_sweep_long (take_long 0) or scanned by
+// the warp that meets them; SHARE: shared out where warps are to spare (compiled
+// in for graphs without such rows, that takes 2% of a sweep of short ones).
+template <int KM, int WK, bool NS, bool SHARE>
+__global__ void __launch_bounds__(kLaneWarps * 32, kLaneBlocks<KM, SHARE>) k_sweep_lane(DevState s, int flag_neighbours, int take_long) {
     using T = typename Acc<WK>::T;
     using Sh = LaneShape<KM, WK>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -512,7 +515,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, kLaneBlocks<KM>) k_sweep_lane
     // second time and take its longer rows, one part of at most 32 entries each
     // (otherwise the rows of a chunk are scanned one after another: 2,000 vertices
     // of degree 90, unit weights, 5 sweeps: 320 us, so 110).
-    const bool shared_out = take_long == 2 && nchunks * 2u <= nwarps;
+    const bool shared_out = SHARE && nchunks * 2u <= nwarps;
     if (shared_out && chunk >= nchunks) {
         const unsigned others = nwarps - nchunks, width = (cnt + others - 1u) / others;     // <= 32
         const unsigned k = (chunk - nchunks) * width + lane;
@@ -739,41 +742,65 @@ static cudaError_t launch_long_k(const DevState& s, int flag, int all, cudaStrea
     return cudaGetLastError();
 }
 
-template <int KM, int WK, bool NS>
-static cudaError_t launch_lane_k(const DevState& s, int flag, cudaStream_t st, int sms, const LaneFork* fork) {
+// Appends the nodes that the next launch captured from st would depend on (none
+// outside a capture, or at the beginning of one).
+static cudaError_t captured_deps(cudaStream_t st, std::vector<cudaGraphNode_t>& deps) {
+    cudaStreamCaptureStatus status;
+    cudaGraph_t graph = nullptr;
+    const cudaGraphNode_t* d = nullptr;
+    size_t n = 0;
+    const cudaError_t err = cudaStreamGetCaptureInfo(st, &status, nullptr, &graph, &d, nullptr, &n);
+    if (err == cudaSuccess && status == cudaStreamCaptureStatusActive) deps.insert(deps.end(), d, d + n);
+    return err;
+}
+
+static cudaError_t set_deps(cudaStream_t st, std::vector<cudaGraphNode_t>& deps) {
+    return cudaStreamUpdateCaptureDependencies(st, deps.data(), nullptr, deps.size(), cudaStreamSetCaptureDependencies);
+}
+
+template <int KM, int WK, bool NS, bool SHARE>
+static cudaError_t launch_lane_k(const DevState& s, int flag, cudaStream_t st, int sms) {
     constexpr int threads = kLaneWarps * 32;
     const bool apart = KM == KEY_PLACE && s.long_rows == 2;
     const size_t smem = kLaneWarps * LaneShape<KM, WK>::WARP_BYTES;
-    auto kern = k_sweep_lane<KM, WK, NS>;
+    auto kern = k_sweep_lane<KM, WK, NS, SHARE>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     int per_sm = 0;
     err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
     if (err != cudaSuccess) return err;
     if (per_sm < 1) per_sm = 1;
-    // the two kernels write different vertices, so a graph runs them side by side
-    // (one after the other, a batch of 64 planted partitions, 3.2 M entries, fp32
-    // weights, lost 4 of 32 us a sweep)
-    const bool beside = apart && fork != nullptr;
-    if (beside) {
-        if ((err = cudaEventRecord(fork->begin, st)) != cudaSuccess) return err;
-        if ((err = cudaStreamWaitEvent(fork->st, fork->begin, 0)) != cudaSuccess) return err;
-    }
-    kern<<<sms * per_sm, threads, smem, st>>>(s, flag, apart ? 0 : s.long_rows ? 2 : 1);
+    // The two kernels write different vertices, so a captured sweep runs them side
+    // by side: the second takes the first one's dependencies, what follows waits
+    // for both (one after the other, a batch of 64 planted partitions, 3.2 M
+    // entries, fp32 weights, lost 4 of 32 us a sweep).
+    std::vector<cudaGraphNode_t> before, both;
+    if (apart && (err = captured_deps(st, before)) != cudaSuccess) return err;
+    kern<<<sms * per_sm, threads, smem, st>>>(s, flag, apart ? 0 : 1);
     err = cudaGetLastError();
     if constexpr (KM == KEY_PLACE) {
-        if (err == cudaSuccess && apart) err = launch_long_k<WK, NS>(s, flag, 0, beside ? fork->st : st, sms);
-    }
-    if (beside) {
-        if (err == cudaSuccess) err = cudaEventRecord(fork->end, fork->st);
-        if (err == cudaSuccess) err = cudaStreamWaitEvent(st, fork->end, 0);
+        if (err != cudaSuccess || !apart) return err;
+        if (before.empty()) return launch_long_k<WK, NS>(s, flag, 0, st, sms);
+        if ((err = captured_deps(st, both)) != cudaSuccess) return err;
+        if ((err = set_deps(st, before)) != cudaSuccess) return err;
+        if ((err = launch_long_k<WK, NS>(s, flag, 0, st, sms)) != cudaSuccess) return err;
+        if ((err = captured_deps(st, both)) != cudaSuccess) return err;
+        err = set_deps(st, both);
     }
     return err;
 }
 
+template <int KM, int WK, bool NS>
+static cudaError_t launch_lane_s(const DevState& s, int flag, cudaStream_t st, int sms) {
+    if constexpr (KM != KEY_PLACE) {
+        if (s.long_rows) return launch_lane_k<KM, WK, NS, true>(s, flag, st, sms);
+    }
+    return launch_lane_k<KM, WK, NS, false>(s, flag, st, sms);
+}
+
 template <int KM, int WK>
-static cudaError_t launch_lane_t(const DevState& s, int flag, int ns, cudaStream_t st, int sms, const LaneFork* fork) {
-    return ns ? launch_lane_k<KM, WK, true>(s, flag, st, sms, fork) : launch_lane_k<KM, WK, false>(s, flag, st, sms, fork);
+static cudaError_t launch_lane_t(const DevState& s, int flag, int ns, cudaStream_t st, int sms) {
+    return ns ? launch_lane_s<KM, WK, true>(s, flag, st, sms) : launch_lane_s<KM, WK, false>(s, flag, st, sms);
 }
 
 // The key layout of the graph's rows, -1 if none fits.
@@ -792,27 +819,27 @@ int lane_long_rows(const DevState& s, int64_t max_degree) {
 }
 
 template <int WK>
-static cudaError_t launch_lane_w(const DevState& s, int flag, int ns, cudaStream_t st, int sms, const LaneFork* fork) {
+static cudaError_t launch_lane_w(const DevState& s, int flag, int ns, cudaStream_t st, int sms) {
     if constexpr (WK == W_UNIT) {
-        return launch_lane_t<KEY_LABEL, WK>(s, flag, ns, st, sms, fork);
+        return launch_lane_t<KEY_LABEL, WK>(s, flag, ns, st, sms);
     } else {
         const int key = key_of(s);
         if constexpr (WK != W_F32) {
-            if (key == KEY_PACKED) return launch_lane_t<KEY_PACKED, WK>(s, flag, ns, st, sms, fork);
+            if (key == KEY_PACKED) return launch_lane_t<KEY_PACKED, WK>(s, flag, ns, st, sms);
         }
-        if (key == KEY_PLACE) return launch_lane_t<KEY_PLACE, WK>(s, flag, ns, st, sms, fork);
+        if (key == KEY_PLACE) return launch_lane_t<KEY_PLACE, WK>(s, flag, ns, st, sms);
         return ns ? launch_long_k<WK, true>(s, flag, 1, st, sms) : launch_long_k<WK, false>(s, flag, 1, st, sms);
     }
 }
 
-cudaError_t launch_sweep_lane(const DevState& s, int mode, cudaStream_t st, int sms, const LaneFork* fork) {
+cudaError_t launch_sweep_lane(const DevState& s, int mode, cudaStream_t st, int sms) {
     const int ns = (mode & kModeNonstrict) != 0;
     const int flag = (mode & ~kModeNonstrict) != MODE_SYNC_FULL;
     switch (s.weight_kind) {
-        case W_UNIT: return launch_lane_w<W_UNIT>(s, flag, ns, st, sms, fork);
-        case W_U32: return launch_lane_w<W_U32>(s, flag, ns, st, sms, fork);
-        case W_U8: return launch_lane_w<W_U8>(s, flag, ns, st, sms, fork);
-        default: return launch_lane_w<W_F32>(s, flag, ns, st, sms, fork);
+        case W_UNIT: return launch_lane_w<W_UNIT>(s, flag, ns, st, sms);
+        case W_U32: return launch_lane_w<W_U32>(s, flag, ns, st, sms);
+        case W_U8: return launch_lane_w<W_U8>(s, flag, ns, st, sms);
+        default: return launch_lane_w<W_F32>(s, flag, ns, st, sms);
     }
 }
 

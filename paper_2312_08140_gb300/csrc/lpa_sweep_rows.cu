@@ -191,8 +191,12 @@ struct RowsShape {
 // for the last bin and two 256-thread blocks for the bin before it ran the
 // run in 107 ms; two and four blocks (64 registers, 4 gathers per thread)
 // took 154 ms, and with 8 gathers per thread (spilling) 136 ms.  The weighted
-// kernels keep 4 gathers per thread either way and take twice the blocks
-// (R-MAT of 769,230 vertices, weights 1..1000: 8.9 -> 8.3 ms).
+// kernels keep 4 gathers per thread either way and take twice the blocks (R-MAT
+// 22, edge factor 12, synchronous / asynchronous: weights 1..1000 70.5 -> 60.8 /
+// 6.5 -> 5.7 ms, fp32 56.1 -> 51.5 / 5.9 -> 5.4; planted partitions of mean degree
+// 1500, fp32 2.96 -> 2.60 ms).  One-byte weights gain no more than they lose
+// (weights 1..4: 4.18 -> 4.20 / 4.31 -> 4.38 ms; mean degree 1500 693 -> 678 us).
+// At 64 registers a thread some of the kernels spill, up to 56 bytes.
 template <int NT, int WK>
 struct RowsOccupancy {
     static constexpr int kBlocks = (NT >= 512 ? 1 : NT >= 256 ? 2 : 8) * (WK != W_UNIT && NT >= 256 ? 2 : 1);

@@ -1,8 +1,7 @@
 // lpa_warp_row.cuh -- a whole warp (or block) on one row: 16-byte reads of a
 // row's ids and its neighbours' marks (row and majority kernels), per-label
 // sums by lane groups and a per-warp open-addressing table in shared memory
-// (warp kernel), and the label sums of a row of more than 32 entries (lane
-// kernel, for the rows it does not sort).
+// (warp kernel), and the label sums of a row that no lane sorts (lane kernels).
 #pragma once
 
 #include "lpa_device.cuh"
